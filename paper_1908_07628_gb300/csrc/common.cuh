@@ -26,6 +26,20 @@ inline cudaError_t smem_attr_once(K* kernel, size_t bytes, std::atomic<uint64_t>
   return e;
 }
 
+// SMs of the current device.
+inline int sm_count() {
+  static std::atomic<int> count[64] = {};
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 148;
+  int c = count[dev].load(std::memory_order_relaxed);
+  if (c == 0) {
+    if (cudaDeviceGetAttribute(&c, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || c <= 0)
+      c = 148;
+    count[dev].store(c, std::memory_order_relaxed);
+  }
+  return c;
+}
+
 __device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
 __device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
 __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
@@ -113,8 +127,7 @@ __device__ __forceinline__ void dft<2, true>(float2* u, unsigned) { float2 a = u
 // Input masks.  The DFTs below take a bit mask `nz` of the inputs that may be nonzero
 // (bit q for input q); inputs outside it must hold zero and the sums and differences
 // with them are skipped.  The masks are compile-time constants once the fully unrolled
-// transforms are inlined, so a pruned butterfly costs nothing at run time.  The first
-// stage of an inverse transform of a band-limited sequence sees half its inputs zero.
+// transforms are inlined, so a pruned butterfly costs nothing at run time.
 //
 // a + b and a - b where na / nb say whether a / b may be nonzero
 __device__ __forceinline__ float2 cadd_nz(float2 a, float2 b, bool na, bool nb) {
@@ -280,16 +293,6 @@ __device__ __forceinline__ void dft<32, false>(float2* u, unsigned nz) { dft_com
 template <>
 __device__ __forceinline__ void dft<32, true>(float2* u, unsigned nz) { dft_composite<8, 4, true>(u, nz); }
 
-// First-stage input mask of an inverse transform whose input is band-limited to
-// |frequency| < N/4: for radix R (a multiple of 4) input q holds frequency b + q N/R with
-// b < N/R, inside the band iff q < R/4 or q >= 3R/4.
-__host__ __device__ constexpr unsigned band_mask(int r) {
-  unsigned m = 0u;
-  for (int q = 0; q < r; ++q)
-    if (4 * q < r || 4 * q >= 3 * r) m |= 1u << q;
-  return m;
-}
-
 // ---------------------------------------------------------------------------
 // Register-resident warp FFT.
 //
@@ -392,7 +395,7 @@ __device__ __forceinline__ void twiddles(float2* w, int ks, const float2* __rest
 // Butterfly slot u = lane + 32 t of a stage with NB butterflies per sequence
 // belongs to sequence u / NB, butterfly u % NB.  Sequence r lives at
 // sbuf + r * ld in the warp's shared buffer.
-template <int N, bool INV, bool REV, int S, bool TAB>
+template <int N, bool INV, bool REV, int S>
 __device__ __forceinline__ void reg_fft_stage(float2* v, float2* sbuf, int ld,
                                               const float2* __restrict__ tw, int lane,
                                               unsigned nz) {
@@ -405,7 +408,7 @@ __device__ __forceinline__ void reg_fft_stage(float2* v, float2* sbuf, int ld,
     const int u = lane + 32 * t;
     if ((ROWS * NB) % 32 == 0 || u < ROWS * NB) {
       const int b = u % NB;
-      if constexpr (TAB && P > 1 && PL::NS == 2) {
+      if constexpr (P > 1 && PL::NS == 2) {
         // second stage of a two-stage plan (P R = N): one table load per twiddle
         // exp(-2 pi i q k / N), stored at q P + k so that a warp reads a contiguous run
         const float2* __restrict__ tab = tw + twiddle_table_offset(N, REV) + b % P;
@@ -450,32 +453,20 @@ __device__ __forceinline__ void reg_fft_stage(float2* v, float2* sbuf, int ld,
       }
     }
     __syncwarp();
-    reg_fft_stage<N, INV, REV, S + 1, TAB>(v, sbuf, ld, tw, lane, ~0u);
+    reg_fft_stage<N, INV, REV, S + 1>(v, sbuf, ld, tw, lane, ~0u);
   }
 }
 
 // Transform the ROWS warp-held sequences.  On entry slot u of v holds
 // x_{u/NB0}[u%NB0 + q N/R0] (R0 = first radix), on exit X in the same form for the
-// last radix.  `tw` is a table built by fill_twiddle_tables for this N.  `nz0` masks
-// the first stage's inputs q that may be nonzero (band_mask for a band-limited input).
-// TAB: a two-stage plan reads its second-stage twiddles from the table (one L1 load
-// each) instead of forming them by products from two loads (about one complex product
-// each); the first suits kernels bound by arithmetic issue, the second kernels bound by
-// L1 / shared-memory wavefronts.
-template <int N, bool INV, bool REV, bool TAB = true>
+// last radix.  `tw` is a table built by fill_twiddle_tables for this N. 
+// `nz0` masks the first stage's inputs q that may be nonzero.  A two-stage plan reads its
+// second-stage twiddles from the table (one L1 load each).
+template <int N, bool INV, bool REV>
 __device__ __forceinline__ void reg_fft(float2* v, float2* sbuf, int ld,
                                         const float2* __restrict__ tw, int lane,
                                         unsigned nz0 = ~0u) {
-  reg_fft_stage<N, INV, REV, 0, TAB>(v, sbuf, ld, tw, lane, nz0);
-}
-
-// Table twiddles for a transform in a wavefront-bound kernel: only where a warp's reads
-// of one factor index take a single wavefront (at most 16 distinct entries) or serve
-// two sequences at once.
-template <int N, bool REV>
-__host__ __device__ constexpr bool table_twiddles_cheap() {
-  using PL = Plan<N, REV>;
-  return PL::NS == 2 && (PL::R(0) <= 16 || PL::per(1) > 1);
+  reg_fft_stage<N, INV, REV, 0>(v, sbuf, ld, tw, lane, nz0);
 }
 
 // ---------------------------------------------------------------------------

@@ -838,19 +838,6 @@ cudaError_t gather_impl(const TcBatch& b, cudaStream_t st) {
   return cudaGetLastError();
 }
 
-int sm_count() {
-  static std::atomic<int> count[64] = {};
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 148;
-  int c = count[dev].load(std::memory_order_relaxed);
-  if (c == 0) {
-    if (cudaDeviceGetAttribute(&c, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || c <= 0)
-      c = 148;
-    count[dev].store(c, std::memory_order_relaxed);
-  }
-  return c;
-}
-
 // Launch of one GEMM over a (gx, gy, gz) tile grid (or its listed tiles): the persistent
 // warp-specialised kernel, one CTA per SM at most.
 template <int MODE, int PREC, int BN>

@@ -10,265 +10,283 @@
 //   row pass    (one warp per row y):  zero-pad kx to N, inverse FFT_x, multiply
 //                by t (or conj t), optionally store the even samples (the N/2
 //                representation used by the S-matrices), forward FFT_x, keep the box.
-//   column pass (one warp per column kx'): FFT_y, keep the box, multiply by the
+//   column pass (one CTA per few columns kx'): FFT_y, keep the box, multiply by the
 //                propagator table (or its conjugate), zero-pad, inverse FFT_y.
 //
 // Scale convention: W holds the true row spectrum; the row pass produces N times
 // the true real-space wave and N times the true row spectrum, and the propagator
 // table carries the 1/N^2 that restores W after the column pass.
+#include <algorithm>
 #include <cmath>
 
 #include "common.cuh"
 #include "internal.h"
+#include "plan_fft.cuh"
 
 namespace eels {
 
 namespace {
 
-constexpr int kRowWarps = 4;   // warps per CTA in the row pass (ROWS rows each)
-constexpr int kColCB = 8;      // columns per CTA in the column pass (one warp each)
+constexpr int kRowWarps = 4;   // warps per CTA of the row pass
 
+// CTAs per SM the row pass is compiled for: 64 registers of data per thread leave room for
+// 16 warps; more warps with fewer registers were slower at every grid (1024: 2.72 us per
+// wave with 16 warps, 2.87 with 20, 3.08 with 24).
 template <int N>
-__device__ __forceinline__ void row_pass_body(const float2* __restrict__ W, float2* __restrict__ Phi,
-                                              const float2* __restrict__ t_slice, int conj_t,
-                                              int store_mode, float2* __restrict__ S, int s_waves,
-                                              int64_t s_stride, int fft_out,
-                                              const float2* __restrict__ tw) {
-  constexpr int NH = N / 2, NQ = N / 4;
-  constexpr int ROWS = RegFFT<N>::ROWS;
-  constexpr int LDR = spad_len(N);
-  using PI = Plan<N, true>;    // inverse transform: reversed radix plan
-  using PF = Plan<N, false>;   // forward transform
-  constexpr int E = RegFFT<N>::E;
-  extern __shared__ float2 smem[];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  float2* sbuf = smem + warp * ROWS * LDR;
-  const int y0 = (blockIdx.x * kRowWarps + warp) * ROWS;   // rows y0 .. y0 + ROWS - 1
-  const int64_t wave = blockIdx.y;
-  float2 v[E];
+__host__ __device__ constexpr int row_ctas() {
+  return pf::Seqs<N>::E > 16 ? 4 : 5;
+}
 
-  // inputs of the inverse x-FFT: the band box, zero-padded to N
-  {
-    constexpr int R0 = PI::R(0), NB0 = N / R0, PER0 = PI::per(0);
-#pragma unroll
-    for (int t = 0; t < PER0; ++t) {
-      const int u = lane + 32 * t;
-      const bool live = (ROWS * NB0) % 32 == 0 || u < ROWS * NB0;
-      const int b = u % NB0;
-      const float2* src = W + (wave * N + y0 + u / NB0) * NH;
-#pragma unroll
-      for (int q = 0; q < R0; ++q) {
-        const int pos = b + q * NB0;
-        float2 x = make_float2(0.f, 0.f);
-        if (live && (q * NB0 < NQ || q * NB0 >= N - NQ)) x = src[pos < NQ ? pos : pos - NH];
-        v[t * R0 + q] = x;
-      }
-    }
-  }
-  reg_fft<N, true, true>(v, sbuf, LDR, tw, lane, band_mask(PI::R(0)));
-
-  // real space: slot u holds N psi(x = u%NBL + q N/RL, y0 + u/NBL)
-  {
-    constexpr int RL = PF::R(0), NBL = N / RL, PERL = PF::per(0);
-#pragma unroll
-    for (int t = 0; t < PERL; ++t) {
-      const int u = lane + 32 * t;
-      if ((ROWS * NBL) % 32 == 0 || u < ROWS * NBL) {
-        const int y = y0 + u / NBL, b = u % NBL;
-        const float2* trow = t_slice + (int64_t)y * N;
-        const bool store = store_mode != 0 && (y & 1) == 0 && wave < s_waves;
-        float2* srow = store ? S + wave * s_stride + (int64_t)(y >> 1) * NH : nullptr;
-#pragma unroll
-        for (int q = 0; q < RL; ++q) {
-          const int x = b + q * NBL;
-          float2 val = v[t * RL + q];
-          if (store && store_mode == 2 && !(x & 1)) srow[x >> 1] = val;
-          const float2 tt = trow[x];
-          val = conj_t ? cmulc(val, tt) : cmul(val, tt);
-          if (store && store_mode == 1 && !(x & 1)) srow[x >> 1] = val;
-          v[t * RL + q] = val;
-        }
-      }
-    }
-  }
-  if (!fft_out) return;
-  __syncwarp();
-  reg_fft<N, false, false>(v, sbuf, LDR, tw, lane);
-  {
-    constexpr int RF = PF::R(PF::NS - 1), NBF = N / RF, PERF = PF::per(PF::NS - 1);
-#pragma unroll
-    for (int t = 0; t < PERF; ++t) {
-      const int u = lane + 32 * t;
-      if ((ROWS * NBF) % 32 == 0 || u < ROWS * NBF) {
-        const int b = u % NBF;
-        float2* dst = Phi + (wave * N + y0 + u / NBF) * NH;
-#pragma unroll
-        for (int q = 0; q < RF; ++q) {
-          if (q * NBF < NQ || q * NBF >= N - NQ) {
-            const int pos = b + q * NBF;
-            dst[pos < NQ ? pos : pos - NH] = v[t * RF + q];
-          }
-        }
-      }
-    }
-  }
+__device__ __forceinline__ void prefetch_l2(const void* p) {
+  asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
 }
 
 template <int N>
-__global__ void __launch_bounds__(kRowWarps * 32)
+struct RowSmem {
+  static constexpr int BUF = pf::Seqs<N>::SEQ * pf::Seqs<N>::PADDED;   // values per warp
+  static constexpr size_t BYTES = (size_t)kRowWarps * BUF * sizeof(float2) +
+                                  (size_t)pf::Seqs<N>::SEQ * N * sizeof(float2) +
+                                  (size_t)pf::SetPart<N>::BOTH * sizeof(float2);
+};
+
+// Row pass.  A CTA takes SEQ rows y0 .. y0 + SEQ - 1 of `chunk` waves, one warp a wave at a
+// time: the rows of t and the factor sets lie in shared memory for all of them (read per
+// row from L2 and L1 they cost as many wavefronts and far more latency), and the rows of a
+// warp's next wave are fetched to L2 while it transforms this one's.  Bound by issue slots
+// (ncu, 1024: 69 %, FMA pipe 55 %, shared-memory wavefronts 66 %, DRAM 45 %).  Adjoint pass
+// with the S_out store, us per wave, before -> now: 1024: 3.22 -> 2.95, 768: 1.83 -> 1.55,
+// 512: 0.58 -> 0.57, 384: 1.00 -> 0.48 (four stages and three exchanges before).
+template <int N, bool CONJ>
+__global__ void __launch_bounds__(kRowWarps * 32, row_ctas<N>())
 k_row_pass(const float2* __restrict__ W, float2* __restrict__ Phi,
-           const float2* __restrict__ t_slice, int conj_t, int store_mode,
-           float2* __restrict__ S, int s_waves, int64_t s_stride, int fft_out,
-           const float2* __restrict__ tw) {
-  row_pass_body<N>(W, Phi, t_slice, conj_t, store_mode, S, s_waves, s_stride, fft_out, tw);
-}
-
-// The 768 plan (radix 24 then 32) would take 132 registers, leaving an SM fewer than 16
-// warps; this form caps it at 128 registers (16 warps per SM) without spills.
-template <int N>
-__global__ void __launch_bounds__(kRowWarps * 32, 16 / kRowWarps)
-k_row_pass_capped(const float2* __restrict__ W, float2* __restrict__ Phi,
-                const float2* __restrict__ t_slice, int conj_t, int store_mode,
-                float2* __restrict__ S, int s_waves, int64_t s_stride, int fft_out,
-                const float2* __restrict__ tw) {
-  row_pass_body<N>(W, Phi, t_slice, conj_t, store_mode, S, s_waves, s_stride, fft_out, tw);
-}
-
-// Padding period of the column tile: the forward transform's first stage reads
-// x[b + q N/R0] from it and the inverse transform's last stage writes the same form.
-template <int N>
-__host__ __device__ constexpr int tile_pad() {
-  return plan2_radix(N, 0) > 0 ? N / plan_radix(N, 0) : 8;
-}
-
-template <int N>
-__host__ __device__ constexpr int col_ld() {
-  // tile column stride: the cooperative tile load / store touches 8*ROWS columns of
-  // one row per half-warp; an odd number of float2 words per column keeps it
-  // conflict-free for 16 columns, 2 mod 16 for 8
-  return spad_len(N) + (rows_per_warp(N) == 2 ? 1 : 2);
-}
-
-template <int N>
-__global__ void __launch_bounds__(kColCB * 32)
-k_col_pass(const float2* __restrict__ Phi, float2* __restrict__ W,
-           const float2* __restrict__ ptab, int conj_p, int mode,
-           const uint8_t* __restrict__ det_mask, const int* __restrict__ wave_out,
-           double* __restrict__ det_acc, double det_scale, const float2* __restrict__ tw) {
+           const float2* __restrict__ t_slice, int store_mode, float2* __restrict__ S,
+           int s_waves, int64_t s_stride, int fft_out, const float2* __restrict__ tw,
+           int n_waves, int chunk) {
   constexpr int NH = N / 2, NQ = N / 4;
-  constexpr int ROWS = RegFFT<N>::ROWS;
-  constexpr int CB = kColCB * ROWS;          // columns per CTA
-  constexpr int LD = col_ld<N>();
-  constexpr int TP = tile_pad<N>();
-  using PI = Plan<N, true>;
-  using PF = Plan<N, false>;
-  constexpr int E = RegFFT<N>::E;
+  constexpr int SEQ = pf::Seqs<N>::SEQ, LD = pf::Seqs<N>::PADDED;
+  using PI = pf::Plan2<N, true>;    // inverse transform: reversed radix plan
+  using PF = pf::Plan2<N, false>;   // forward transform
   extern __shared__ float2 smem[];
+  float2* trows = smem + kRowWarps * RowSmem<N>::BUF;   // [SEQ][N]
+  float2* sets = trows + SEQ * N;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int kx0 = blockIdx.x * CB;
-  const int64_t wave = blockIdx.y;
-  const float2* src = Phi + wave * (int64_t)N * NH;
-  {
-    // all N / (256 / CB) loads of a thread in flight at once
-    const int c = threadIdx.x % CB;
-    constexpr int STEP = (kColCB * 32) / CB, NL = N / STEP;
-    float2 tmp[NL];
+  float2* sbuf = smem + warp * RowSmem<N>::BUF;
+  const int y0 = blockIdx.x * SEQ;
+  const int w0 = blockIdx.y * chunk + warp, w_end = min(n_waves, (int)(blockIdx.y + 1) * chunk);
+  pf::load_sets<N>(sets, tw, false);
+  pf::copy_async(trows, t_slice + (int64_t)y0 * N, SEQ * N);
+
+  float2 v[pf::Seqs<N>::E];
+  // inputs of the inverse x-FFT: the band box, zero-padded to N
+  auto load = [&](int64_t base) {
 #pragma unroll
-    for (int i = 0; i < NL; ++i) tmp[i] = src[(int64_t)(threadIdx.x / CB + i * STEP) * NH + kx0 + c];
+    for (int t = 0; t < PI::PER0; ++t) {
+      const int u = lane + 32 * t;
+      if ((SEQ * PI::NB0) % 32 == 0 || u < SEQ * PI::NB0) {
+        const float2* src = W + base + (u / PI::NB0) * NH + u % PI::NB0;
 #pragma unroll
-    for (int i = 0; i < NL; ++i) smem[c * LD + spad<TP>(threadIdx.x / CB + i * STEP)] = tmp[i];
-  }
+        for (int q = 0; q < PI::R0; ++q) {
+          const int at = q * PI::NB0;
+          if (at < NQ) v[t * PI::R0 + q] = src[at];
+          else if (at >= N - NQ) v[t * PI::R0 + q] = src[at - NH];
+          else v[t * PI::R0 + q] = make_float2(0.f, 0.f);
+        }
+      }
+    }
+  };
+  if (w0 < w_end) load(((int64_t)w0 * N + y0) * NH);
+  pf::cp_async_wait();
   __syncthreads();
-  float2* sbuf = smem + warp * ROWS * LD;    // this warp's ROWS columns
-  float2 v[E];
-  {
-    constexpr int R0 = PF::R(0), NB0 = N / R0, PER0 = PF::per(0);
+
+  for (int64_t wave = w0; wave < w_end; wave += kRowWarps) {
+    const int64_t base = (wave * N + y0) * NH;
+    if (wave != w0) load(base);
+    if (wave + kRowWarps < w_end) {   // the next rows: SEQ * NH values, contiguous
+      const float2* next = W + base + (int64_t)kRowWarps * N * NH;
 #pragma unroll
-    for (int t = 0; t < PER0; ++t) {
+      for (int i = lane * 16; i < SEQ * NH; i += 512) prefetch_l2(next + i);
+    }
+    pf::warp_fft<N, true, true, true>(v, sbuf, LD, pf::rev_set<N>(sets), lane);
+
+    // real space: slot u holds N psi(x = u % NB0 + q N/R0, y0 + u / NB0)
+#pragma unroll
+    for (int t = 0; t < PF::PER0; ++t) {
       const int u = lane + 32 * t;
-      if ((ROWS * NB0) % 32 == 0 || u < ROWS * NB0) {
-        const int b = u % NB0;
-        const float2* col = sbuf + (u / NB0) * LD;
+      if ((SEQ * PF::NB0) % 32 == 0 || u < SEQ * PF::NB0) {
+        const int y = y0 + u / PF::NB0, b = u % PF::NB0;
+        const float2* trow = trows + (u / PF::NB0) * N + b;
+        // even x only: N/R0 is even, so x has the parity of b
+        const bool store = store_mode != 0 && ((y | b) & 1) == 0 && wave < s_waves;
+        float2* srow = S + wave * s_stride + (int64_t)(y >> 1) * NH + (b >> 1);
 #pragma unroll
-        for (int q = 0; q < R0; ++q) v[t * R0 + q] = col[spad<TP>(b + q * NB0)];
+        for (int q = 0; q < PF::R0; ++q) {
+          const float2 before = v[t * PF::R0 + q];
+          const float2 after = pf::mul_c<CONJ>(before, trow[q * PF::NB0]);
+          if (store) srow[q * (PF::NB0 / 2)] = store_mode == 1 ? after : before;
+          v[t * PF::R0 + q] = after;
+        }
+      }
+    }
+    if (!fft_out) continue;
+    pf::warp_fft<N, false, false, false>(v, sbuf, LD, sets, lane);
+#pragma unroll
+    for (int t = 0; t < PF::PER1; ++t) {
+      const int u = lane + 32 * t;
+      if ((SEQ * PF::NB1) % 32 == 0 || u < SEQ * PF::NB1) {
+        float2* dst = Phi + base + (u / PF::NB1) * NH + u % PF::NB1;
+#pragma unroll
+        for (int q = 0; q < PF::R1; ++q) {
+          const int at = q * PF::NB1;
+          if (at < NQ) dst[at] = v[t * PF::R1 + q];
+          else if (at >= N - NQ) dst[at - NH] = v[t * PF::R1 + q];
+        }
       }
     }
   }
-  __syncwarp();
-  // the column pass is bound by wavefronts as much as by arithmetic
-  reg_fft<N, false, false, table_twiddles_cheap<N, false>()>(v, sbuf, LD, tw, lane);
-  // y-spectrum: slot u holds ky = u%NBF + q N/RF of column kx0 + warp*ROWS + u/NBF
-  constexpr int RF = PF::R(PF::NS - 1), NBF = N / RF, PERF = PF::per(PF::NS - 1);
-  if (mode == 0) {
+}
+
+// Column pass.  A CTA takes CB neighbouring columns of `chunk` waves, a wave at a time; a
+// thread holds a butterfly of one column, and the lanes of a warp run over the columns
+// first, so that rows are read and written in segments of CB values straight from
+// registers and shared memory carries only the exchange inside each transform.  (One warp
+// per column with the tile staged in shared memory, the form before, took twice the
+// wavefronts and was bound by them.)  Measured, us per wave, before -> now: 1024: 2.41 ->
+// 1.91, 768: 1.69 -> 1.06, 512: 0.466 -> 0.387, 384: 0.66 -> 0.28, 256: 0.118 -> 0.106; the
+// copy bandwidth would allow 1.23, 0.69, 0.31, 0.17 and 0.08.  CB and CTAs per SM are the
+// fastest measured: 16 columns (128-byte segments) for the grids whose CTA then fills half
+// of an SM's warps by itself, 8 elsewhere.
+template <int N>
+struct ColCfg {
+  using PF = pf::Plan2<N, false>;
+  static constexpr int CB = N == 512 || N == 1024 ? 16 : 8;
+  static constexpr int CTAS = N == 64 ? 8 : N == 128 || N == 256 ? 5 : N == 384 ? 3 : N == 768 ? 2 : 1;
+  static constexpr int TPC = pf::col_threads(N), THREADS = CB * TPC;
+  static constexpr int PER0 = (PF::NB0 + TPC - 1) / TPC, PER1 = (PF::NB1 + TPC - 1) / TPC;
+  static constexpr int E = PER0 * PF::R0 > PER1 * PF::R1 ? PER0 * PF::R0 : PER1 * PF::R1;
+  static constexpr int EX = pf::Seqs<N>::PADDED * CB;   // exchange buffer, values
+  static constexpr size_t BYTES = (size_t)(EX + pf::SetPart<N>::BOTH) * sizeof(float2);
+};
+
+// MODE 0 / 1: multiply by the propagator table / its conjugate and go back to rows;
+// MODE 2: multiply by the table and sum |.|^2 over the detector bins.
+template <int N, int MODE>
+__global__ void __launch_bounds__(ColCfg<N>::THREADS, ColCfg<N>::CTAS)
+k_col_pass(const float2* __restrict__ Phi, float2* __restrict__ W, const float2* __restrict__ ptab,
+           const uint8_t* __restrict__ det_mask, const int* __restrict__ wave_out,
+           double* __restrict__ det_acc, double det_scale, const float2* __restrict__ tw,
+           int n_waves, int chunk) {
+  using CC = ColCfg<N>;
+  constexpr int NH = N / 2, NQ = N / 4, CB = CC::CB;
+  using PF = pf::Plan2<N, false>;
+  using PI = pf::Plan2<N, true>;
+  constexpr bool EXACT = pf::exact_factors(N, true);
+  extern __shared__ float2 ex[];
+  float2* fset = ex + CC::EX;
+  const float2* rset = pf::rev_set<N>(fset);
+  const int c = threadIdx.x % CB, b0 = threadIdx.x / CB;
+  const int kx = blockIdx.x * CB + c;
+  const int w0 = blockIdx.y * chunk, w_end = min(n_waves, (int)(blockIdx.y + 1) * chunk);
+  pf::load_sets<N>(fset, tw, true);
+  using SP = pf::SetPart<N>;
+
+  for (int64_t wave = w0; wave < w_end; ++wave) {
+    float2 v[CC::E];
+    const float2* src = Phi + wave * N * NH + kx;
 #pragma unroll
-    for (int t = 0; t < PERF; ++t) {
-      const int u = lane + 32 * t;
-      const bool live = (ROWS * NBF) % 32 == 0 || u < ROWS * NBF;
-      const int b = u % NBF;
-      const float2* prow = ptab + (int64_t)(kx0 + warp * ROWS + u / NBF) * NH;
+    for (int t = 0; t < CC::PER0; ++t) {
+      const int b = b0 + t * CC::TPC;
+      if (PF::NB0 % CC::TPC == 0 || b < PF::NB0) {
 #pragma unroll
-      for (int q = 0; q < RF; ++q) {
-        float2 val = make_float2(0.f, 0.f);
-        if (live && (q * NBF < NQ || q * NBF >= N - NQ)) {
-          const int pos = b + q * NBF;
-          const float2 p = prow[pos < NQ ? pos : pos - NH];
-          val = conj_p ? cmulc(v[t * RF + q], p) : cmul(v[t * RF + q], p);
-        }
-        v[t * RF + q] = val;
+        for (int q = 0; q < PF::R0; ++q)
+          v[t * PF::R0 + q] = src[(int64_t)(b + q * PF::NB0) * NH];
       }
     }
-    __syncwarp();
-    reg_fft<N, true, true, table_twiddles_cheap<N, true>()>(v, sbuf, LD, tw, lane,
-                                                           band_mask(PI::R(0)));
-    {
-      constexpr int RL = PI::R(PI::NS - 1), NBL = N / RL, PERL = PI::per(PI::NS - 1);
+    if (N > 256 && wave + 1 < w_end) {   // the next wave's rows of these columns
+      const float2* next = Phi + ((wave + 1) * N + threadIdx.x) * NH + blockIdx.x * CB;
 #pragma unroll
-      for (int t = 0; t < PERL; ++t) {
-        const int u = lane + 32 * t;
-        if ((ROWS * NBL) % 32 == 0 || u < ROWS * NBL) {
-          const int b = u % NBL;
-          float2* col = sbuf + (u / NBL) * LD;
+      for (int r = 0; r < N / CC::THREADS; ++r) prefetch_l2(next + (int64_t)r * CC::THREADS * NH);
+    }
+    pf::cp_async_wait();
+    __syncthreads();   // the factor sets are there; the last exchange has been read
 #pragma unroll
-          for (int q = 0; q < RL; ++q) col[spad<TP>(b + q * NBL)] = v[t * RL + q];
-        }
+    for (int t = 0; t < CC::PER0; ++t) {
+      const int b = b0 + t * CC::TPC;
+      if (PF::NB0 % CC::TPC == 0 || b < PF::NB0) {
+        pf::super_stage<PF::A0, PF::B0, 1, false, false, EXACT>(v + t * PF::R0, 0, nullptr,
+                                                                fset + SP::AT0);
+        float2* dst = ex + b * (PF::R0 + 1) * CB + c;
+#pragma unroll
+        for (int o = 0; o < PF::R0; ++o) dst[o * CB] = v[t * PF::R0 + o];
       }
     }
     __syncthreads();
-    float2* dst = W + wave * (int64_t)N * NH;
-    const int c = threadIdx.x % CB;
-    constexpr int STEP = (kColCB * 32) / CB, NL = N / STEP;
 #pragma unroll
-    for (int i = 0; i < NL; ++i) {
-      const int r = threadIdx.x / CB + i * STEP;
-      dst[(int64_t)r * NH + kx0 + c] = smem[c * LD + spad<TP>(r)];
+    for (int t = 0; t < CC::PER1; ++t) {
+      const int b = b0 + t * CC::TPC;
+      if (PF::NB1 % CC::TPC == 0 || b < PF::NB1) {
+        const float2* from = ex + b * CB + c;
+#pragma unroll
+        for (int q = 0; q < PF::R1; ++q) v[t * PF::R1 + q] = from[q * (PF::NB1 + 1) * CB];
+      }
     }
-  } else {
-    const int out = wave_out[wave];
-    if (out < 0) return;
+    if constexpr (MODE != 2) __syncthreads();   // read before the inverse overwrites it
     float acc = 0.f;
 #pragma unroll
-    for (int t = 0; t < PERF; ++t) {
-      const int u = lane + 32 * t;
-      const bool live = (ROWS * NBF) % 32 == 0 || u < ROWS * NBF;
-      const int b = u % NBF;
-      const int kx = kx0 + warp * ROWS + u / NBF;
-      const float2* prow = ptab + (int64_t)kx * NH;
-      const uint8_t* mrow = det_mask + (int64_t)kx * NH;
+    for (int t = 0; t < CC::PER1; ++t) {
+      const int b = b0 + t * CC::TPC;
+      if (PF::NB1 % CC::TPC == 0 || b < PF::NB1) {
+        float2* x = v + t * PF::R1;
+        pf::super_stage<PF::A1, PF::B1, PF::R0, false, false, EXACT>(x, b, fset + SP::AT1,
+                                                                     fset + SP::AT2);
+        // x[q] is ky = b + q NB1; the table depends on kx^2 + ky^2 only, so its rows may be
+        // read along kx
 #pragma unroll
-      for (int q = 0; q < RF; ++q) {
-        if (live && (q * NBF < NQ || q * NBF >= N - NQ)) {
-          const int pos = b + q * NBF;
-          const int ky = pos < NQ ? pos : pos - NH;
-          if (mrow[ky]) {
-            const float2 val = conj_p ? cmulc(v[t * RF + q], prow[ky]) : cmul(v[t * RF + q], prow[ky]);
-            acc = fmaf(val.x, val.x, fmaf(val.y, val.y, acc));
+        for (int q = 0; q < PF::R1; ++q) {
+          const int at = q * PF::NB1;
+          if (at < NQ || at >= N - NQ) {
+            const int ky = b + (at < NQ ? at : at - NH);
+            if constexpr (MODE != 2) {
+              x[q] = pf::mul_c<MODE == 1>(x[q], __ldg(ptab + (int64_t)ky * NH + kx));
+            } else if (det_mask[(int64_t)kx * NH + ky]) {
+              const float2 val = pf::mul(x[q], __ldg(ptab + (int64_t)ky * NH + kx));
+              acc = fmaf(val.x, val.x, fmaf(val.y, val.y, acc));
+            }
+          } else {
+            x[q] = make_float2(0.f, 0.f);
           }
+        }
+        if constexpr (MODE != 2) {
+          pf::super_stage<PI::A0, PI::B0, 1, true, true, EXACT>(x, 0, nullptr, rset + SP::AT0);
+          float2* dst = ex + b * (PI::R0 + 1) * CB + c;
+#pragma unroll
+          for (int o = 0; o < PI::R0; ++o) dst[o * CB] = x[o];
         }
       }
     }
+    if constexpr (MODE != 2) {
+      __syncthreads();
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (lane == 0 && acc != 0.f) atomicAdd(det_acc + out, det_scale * (double)acc);
+      for (int t = 0; t < CC::PER0; ++t) {
+        const int b = b0 + t * CC::TPC;
+        if (PI::NB1 % CC::TPC == 0 || b < PI::NB1) {
+          float2* x = v + t * PI::R1;
+          const float2* from = ex + b * CB + c;
+#pragma unroll
+          for (int q = 0; q < PI::R1; ++q) x[q] = from[q * (PI::NB1 + 1) * CB];
+          pf::super_stage<PI::A1, PI::B1, PI::R0, true, false, EXACT>(x, b, rset + SP::AT1,
+                                                                      rset + SP::AT2);
+          float2* dst = W + (wave * N + b) * NH + kx;
+#pragma unroll
+          for (int q = 0; q < PI::R1; ++q) dst[(int64_t)q * PI::NB1 * NH] = x[q];
+        }
+      }
+    } else {
+      const int out = wave_out[wave];
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+      if ((threadIdx.x & 31) == 0 && out >= 0 && acc != 0.f)
+        atomicAdd(det_acc + out, det_scale * (double)acc);
+    }
   }
 }
 
@@ -427,21 +445,53 @@ __global__ void k_spawn(int n, const int* __restrict__ src, const int* __restric
   }
 }
 
+// Waves per CTA: a multiple of the waves in flight in it (`width`), at most 16 of them, and
+// no more than leave about kCtaRounds CTAs per resident one (`resident`: CTAs the device holds).
+constexpr int kCtaRounds = 3;
+int wave_chunk(int n_waves, int blocks_x, int width, int resident) {
+  const int64_t items = (n_waves + width - 1) / width;
+  const int64_t per = std::max<int64_t>(1, items * blocks_x / (kCtaRounds * (int64_t)resident));
+  return width * (int)std::min<int64_t>(per, 16);
+}
+
+template <int N, bool CONJ>
+cudaError_t row_pass_c(int n_waves, const float2* W, float2* Phi, const float2* t, int store_mode,
+                       float2* S, int s_waves, int64_t s_stride, int fft_out, const float2* tw,
+                       cudaStream_t s) {
+  static std::atomic<uint64_t> attr{0};
+  cudaError_t e = smem_attr_once(k_row_pass<N, CONJ>, RowSmem<N>::BYTES, attr);
+  if (e != cudaSuccess) return e;
+  const int gx = N / pf::Seqs<N>::SEQ;
+  const int chunk = wave_chunk(n_waves, gx, kRowWarps, sm_count() * row_ctas<N>());
+  dim3 grid(gx, (n_waves + chunk - 1) / chunk);
+  k_row_pass<N, CONJ><<<grid, kRowWarps * 32, RowSmem<N>::BYTES, s>>>(
+      W, Phi, t, store_mode, S, s_waves, s_stride, fft_out, tw, n_waves, chunk);
+  return cudaGetLastError();
+}
+
 template <int N>
 cudaError_t row_pass_n(int n_waves, const float2* W, float2* Phi, const float2* t, int conj_t,
                        int store_mode, float2* S, int s_waves, int64_t s_stride, int fft_out,
                        const float2* tw, cudaStream_t s) {
-  constexpr int ROWS = RegFFT<N>::ROWS;
-  const size_t smem = (size_t)kRowWarps * ROWS * spad_len(N) * sizeof(float2);
-  auto kern = [] {
-    if constexpr (N == 768) return k_row_pass_capped<N>;
-    else return k_row_pass<N>;
-  }();
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  return conj_t ? row_pass_c<N, true>(n_waves, W, Phi, t, store_mode, S, s_waves, s_stride,
+                                      fft_out, tw, s)
+                : row_pass_c<N, false>(n_waves, W, Phi, t, store_mode, S, s_waves, s_stride,
+                                       fft_out, tw, s);
+}
+
+template <int N, int MODE>
+cudaError_t col_pass_m(int n_waves, const float2* Phi, float2* W, const float2* ptab,
+                       const uint8_t* det_mask, const int* wave_out, double* det_acc,
+                       double det_scale, const float2* tw, cudaStream_t s) {
+  using CC = ColCfg<N>;
+  static std::atomic<uint64_t> attr{0};
+  cudaError_t e = smem_attr_once(k_col_pass<N, MODE>, CC::BYTES, attr);
   if (e != cudaSuccess) return e;
-  dim3 grid(N / (kRowWarps * ROWS), n_waves);
-  kern<<<grid, kRowWarps * 32, smem, s>>>(W, Phi, t, conj_t, store_mode, S, s_waves, s_stride,
-                                          fft_out, tw);
+  const int gx = N / 2 / CC::CB;
+  const int chunk = wave_chunk(n_waves, gx, 1, sm_count() * CC::CTAS);
+  dim3 grid(gx, (n_waves + chunk - 1) / chunk);
+  k_col_pass<N, MODE><<<grid, CC::THREADS, CC::BYTES, s>>>(
+      Phi, W, ptab, det_mask, wave_out, det_acc, det_scale, tw, n_waves, chunk);
   return cudaGetLastError();
 }
 
@@ -449,15 +499,12 @@ template <int N>
 cudaError_t col_pass_n(int n_waves, const float2* Phi, float2* W, const float2* ptab, int conj_p,
                        int mode, const uint8_t* det_mask, const int* wave_out, double* det_acc,
                        double det_scale, const float2* tw, cudaStream_t s) {
-  constexpr int ROWS = RegFFT<N>::ROWS;
-  const size_t smem = (size_t)kColCB * ROWS * col_ld<N>() * sizeof(float2);
-  cudaError_t e = cudaFuncSetAttribute(k_col_pass<N>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       (int)smem);
-  if (e != cudaSuccess) return e;
-  dim3 grid(N / 2 / (kColCB * ROWS), n_waves);
-  k_col_pass<N><<<grid, kColCB * 32, smem, s>>>(Phi, W, ptab, conj_p, mode, det_mask, wave_out,
-                                                det_acc, det_scale, tw);
-  return cudaGetLastError();
+  if (mode == 1)
+    return col_pass_m<N, 2>(n_waves, Phi, W, ptab, det_mask, wave_out, det_acc, det_scale, tw, s);
+  return conj_p ? col_pass_m<N, 1>(n_waves, Phi, W, ptab, det_mask, wave_out, det_acc, det_scale,
+                                   tw, s)
+                : col_pass_m<N, 0>(n_waves, Phi, W, ptab, det_mask, wave_out, det_acc, det_scale,
+                                   tw, s);
 }
 
 }  // namespace
@@ -471,7 +518,65 @@ bool grid_supported(int n) {
   return false;
 }
 
-int twiddle_table_size(int n) { return twiddle_table_len(n); }
+int twiddle_table_size(int n) {
+  return grid_supported(n) ? pf::table_len(n) : twiddle_table_len(n);
+}
+
+namespace {
+
+// Factors of one set of the plans of plan_fft.cuh.
+void fill_plan_set(int n, bool col, bool rev, float2* h) {
+  const float2* root = h;   // exp(-2 pi i k / n), k < n
+  float2* set = h + pf::set_offset(n, col, rev);
+  const int a0 = pf::plan_a(n, rev, 0), b0 = pf::plan_b(n, rev, 0);
+  const int a1 = pf::plan_a(n, rev, 1), b1 = pf::plan_b(n, rev, 1);
+  for (int i = 0; i < pf::set_len(n); ++i) set[i] = make_float2(0.f, 0.f);
+  auto mul = [](float2 a, float2 b) {   // the rounding of the device's cmul
+    return make_float2(std::fmaf(a.x, b.x, -(a.y * b.y)), std::fmaf(a.x, b.y, a.y * b.x));
+  };
+  // the radix-r factors exp(-2 pi i q ks / n), q < r: table entries, or for r > 4 products
+  // of two of them
+  auto factors = [&](int r, int ks, float2* w) {
+    w[0] = make_float2(1.f, 0.f);
+    if (r <= 4) {
+      for (int q = 1; q < r; ++q) w[q] = root[(q * ks) % n];
+      return;
+    }
+    w[1] = root[ks];
+    w[2] = mul(w[1], w[1]);
+    w[3] = mul(w[2], w[1]);
+    w[4] = mul(w[2], w[2]);
+    for (int q = 5; q < std::min(r, 8); ++q) w[q] = mul(w[4], w[q - 4]);
+    float2 hi = root[(8 * ks) % n];
+    const float2 w8 = hi;
+    for (int a = 1; a < r / 8; ++a) {
+      w[8 * a] = hi;
+      for (int q = 1; q < 8; ++q) w[8 * a + q] = mul(hi, w[q]);
+      hi = mul(hi, w8);
+    }
+  };
+  float2 w[32];
+  if (b0 > 1)
+    for (int k = 0; k < a0; ++k) {
+      factors(b0, k * (n / (a0 * b0)), w);
+      for (int m = 0; m < b0; ++m) set[m * a0 + k] = w[m];
+    }
+  const int p = a0 * b0, p1 = p * a1;
+  for (int k = 0; k < p; ++k) {
+    if (pf::exact_factors(n, col))
+      for (int q = 0; q < a1; ++q) w[q] = root[(q * k) % n];
+    else
+      factors(a1, k * (n / p1), w);
+    for (int q = 0; q < a1; ++q) set[32 + q * p + k] = w[q];
+  }
+  if (b1 > 1)
+    for (int k = 0; k < p1; ++k) {
+      factors(b1, k * (n / (p1 * b1)), w);
+      for (int m = 0; m < b1; ++m) set[32 + n + m * p1 + k] = w[m];
+    }
+}
+
+}  // namespace
 
 void fill_twiddle_tables(int n, float2* h) {
   auto root = [n](int64_t e) {
@@ -480,6 +585,8 @@ void fill_twiddle_tables(int n, float2* h) {
   };
   for (int k = 0; k < n; ++k) h[k] = root(k);
   for (int k = n; k < twiddle_table_len(n); ++k) h[k] = make_float2(0.f, 0.f);
+  if (grid_supported(n))
+    for (int i = 0; i < 4; ++i) fill_plan_set(n, i >= 2, i & 1, h);
   if (plan_len(n) != 2) return;
   for (int rev = 0; rev < 2; ++rev) {
     // stage 1 of the plan: radix r1 after a first stage of radix r0 (r0 r1 = n)
