@@ -706,19 +706,14 @@ eels_status map_window(eels_ctx* ctx, const eels_smatrix* sm, const eels_transit
   float2* tw = nullptr;
   if ((r = twiddles(ctx, n, &tw)) != EELS_OK) return r;
 
-  // PRISM windows and the transitions of each slice (sites reached by some probe)
+  // PRISM windows and the sites of each slice that some probe reaches
   SiteLists L = window_lists(tr, sc, win, sm->cell, f);
-  std::vector<std::vector<int>> tr_site(n_z), tr_type(n_z);
-  for (int s = 0; s < S; ++s) {
-    if (L.xcnt[s] == 0 || L.ycnt[s] == 0) continue;
-    for (int m = 0; m < T; ++m) {
-      tr_site[tr->slice[s]].push_back(s);
-      tr_type[tr->slice[s]].push_back(m);
-    }
-  }
+  std::vector<std::vector<int>> slice_sites(n_z);
+  for (int s = 0; s < S; ++s)
+    if (L.xcnt[s] > 0 && L.ycnt[s] > 0) slice_sites[tr->slice[s]].push_back(s);
 
-  DevBuf<float2> dH, Sout, W, Phi, M, ax, ay, damp;
-  DevBuf<int> dwx, dwy, dxoff, dxcnt, dxlist, dyoff, dycnt, dylist, dpx, dpy, dbp, dbq, dts, dtt;
+  DevBuf<float2> dH, Sout, W, Phi, M, axT, ayT, damp;
+  DevBuf<int> dwx, dwy, dxoff, dxcnt, dxlist, dyoff, dycnt, dylist, dpx, dpy, dbp, dbq;
   DevBuf<double> dmap;
   const float2* H = (const float2*)tr->H;
   const int h_mul = tr->h_shared ? 0 : 1;
@@ -748,32 +743,25 @@ eels_status map_window(eels_ctx* ctx, const eels_smatrix* sm, const eels_transit
   EELS_CK(dylist.upload(L.ylist.data(), L.ylist.size(), st));
   EELS_CK(dbp.upload(sm->bp.data(), n_in, st));
   EELS_CK(dbq.upload(sm->bq.data(), n_in, st));
-  EELS_CK(ax.alloc((size_t)n_in * win.nx, st));
-  EELS_CK(ay.alloc((size_t)n_in * win.ny, st));
-  EELS_CK(eels::launch_phase_table(ax.p, dbp.p, n_in, f, sm->cell, sc->x0, sc->step_x, win.nx, st,
-                                   0, win.ix0));
-  EELS_CK(eels::launch_phase_table(ay.p, dbq.p, n_in, f, sm->cell, sc->y0, sc->step_y, win.ny, st,
-                                   0, win.iy0));
-  DevBuf<float2> axT, ayT;   // [pos][n_in]: the tensor-core gathers read along the beams
-  if (tc) {
-    EELS_CK(axT.alloc((size_t)n_in * win.nx, st));
-    EELS_CK(ayT.alloc((size_t)n_in * win.ny, st));
-    EELS_CK(eels::launch_phase_table(axT.p, dbp.p, n_in, f, sm->cell, sc->x0, sc->step_x,
-                                     win.nx, st, 1, win.ix0));
-    EELS_CK(eels::launch_phase_table(ayT.p, dbq.p, n_in, f, sm->cell, sc->y0, sc->step_y,
-                                     win.ny, st, 1, win.iy0));
-  }
+  // phase tables [pos][n_in]: the contractions read along the beams
+  EELS_CK(axT.alloc((size_t)n_in * win.nx, st));
+  EELS_CK(ayT.alloc((size_t)n_in * win.ny, st));
+  EELS_CK(eels::launch_phase_table(axT.p, dbp.p, n_in, f, sm->cell, sc->x0, sc->step_x, win.nx,
+                                   st, 1, win.ix0));
+  EELS_CK(eels::launch_phase_table(ayT.p, dbq.p, n_in, f, sm->cell, sc->y0, sc->step_y, win.ny,
+                                   st, 1, win.iy0));
 
-  // flattened transition lists of all slices
-  std::vector<int> all_site, all_type, slice_off(n_z + 1, 0);
+  // reached sites of all slices, slice after slice
+  std::vector<int> slot_all, site_off(n_z + 1, 0);
+  int max_sites = 0;
   for (int i = 0; i < n_z; ++i) {
-    slice_off[i] = (int)all_site.size();
-    all_site.insert(all_site.end(), tr_site[i].begin(), tr_site[i].end());
-    all_type.insert(all_type.end(), tr_type[i].begin(), tr_type[i].end());
+    site_off[i] = (int)slot_all.size();
+    slot_all.insert(slot_all.end(), slice_sites[i].begin(), slice_sites[i].end());
+    max_sites = std::max(max_sites, (int)slice_sites[i].size());
   }
-  slice_off[n_z] = (int)all_site.size();
-  EELS_CK(dts.upload(all_site.data(), all_site.size(), st));
-  EELS_CK(dtt.upload(all_type.data(), all_type.size(), st));
+  site_off[n_z] = (int)slot_all.size();
+  DevBuf<int> dslot;
+  EELS_CK(dslot.upload(slot_all.data(), slot_all.size(), st));
 
   // detector plane waves at the exit surface, carried back by conj(P) first:
   // beta_d(n_z - 1) = conj(P(k_d)) |k_d>
@@ -806,22 +794,20 @@ eels_status map_window(eels_ctx* ctx, const eels_smatrix* sm, const eels_transit
     EELS_CK(seg.alloc((size_t)K * n_in * plane, st));
   }
 
-  // M buffer: a batch of transitions, at most ~1 GiB
+  // M buffer of the FP32 path, at most ~1 GiB of transitions: all types of a batch of
+  // sites, or some types of one site
   const int64_t m_stride = (int64_t)n_out * n_in;
-  int max_tr = 0;
-  for (int i = 0; i < n_z; ++i) max_tr = std::max(max_tr, (int)tr_site[i].size());
-  const int batch = (int)std::max<int64_t>(1, std::min<int64_t>(
-      std::max(max_tr, 1), (int64_t)(1 << 30) / (m_stride * (int64_t)sizeof(float2))));
-  if (!tc) EELS_CK(M.alloc((size_t)batch * m_stride, st));
+  const int64_t m_cap = std::max<int64_t>(1, ((int64_t)1 << 30) / (m_stride * (int64_t)sizeof(float2)));
+  const int fp_types = (int)std::min<int64_t>(T, m_cap);
+  const int fp_sites = fp_types < T ? 1 : (int)std::min<int64_t>(
+      std::min(std::max(max_sites, 1), 65535), m_cap / T);
+  if (!tc) EELS_CK(M.alloc((size_t)fp_sites * fp_types * m_stride, st));
 
   // tensor-core path: sites of a slice in batches of `sb` slots
   auto rup = [](int64_t v, int64_t m) { return (v + m - 1) / m * m; };
   const int kal = eels::tc_k_align(tc_prec);
   const int k1p = (int)rup(2 * (int64_t)w * w, kal), k2p = (int)rup(2 * (int64_t)n_in, kal);
   const int nr_cap = std::max(L.max_nr, 1);
-  std::vector<std::vector<int>> slice_sites(n_z);
-  for (int s = 0; s < S; ++s)
-    if (L.xcnt[s] > 0 && L.ycnt[s] > 0) slice_sites[tr->slice[s]].push_back(s);
   // AUTO: measured once per shape (both groupings timed on the first occupied slice)
   const std::vector<int64_t> shape_key = {tc_prec, n, n_out, n_in, w, nr_cap, T};
   int chosen = ctx->assoc;
@@ -883,31 +869,24 @@ eels_status map_window(eels_ctx* ctx, const eels_smatrix* sm, const eels_transit
            (need_tr ? (int64_t)T * 2 * n_in * k1p + (int64_t)T * n_out * k2p +
                           (int64_t)2 * nr_cap * k2p
                     : 0));
-  int max_sites = 0;
-  for (int i = 0; i < n_z; ++i) max_sites = std::max(max_sites, (int)slice_sites[i].size());
   int sb = (int)std::max<int64_t>(1, std::min<int64_t>(std::max(max_sites, 1),
                                                        ctx->operand_budget / per_site));
   if (ctx->batch_sites > 0) sb = std::min(sb, ctx->batch_sites);
   DevBuf<float> A1, B1, M1, B2, AY, BY, BV;
-  DevBuf<int> dslot, dzs, dzt, dab1, dbb1, dnv1, dab2, dbb2, dnv2, dstatus, daby, dnvy, dnry;
+  DevBuf<int> dzs, dzt, dab1, dbb1, dnv1, dab2, dbb2, dnv2, dstatus, daby, dnvy, dnry;
   DevBuf<double> dscratch;
-  std::vector<int> slot_all, zs_all, zt_all, nv2_all, nr_all, site_off(n_z + 1, 0);
+  std::vector<int> zs_all, zt_all, nv2_all, nr_all;
   std::vector<int> pv_all[2], py_all[2];   // [0]: 256-column tiles, [1]: 128-column tiles
   DevBuf<int> dtile_v[2], dtile_y[2];
   if (tc) {
-    for (int i = 0; i < n_z; ++i) {
-      site_off[i] = (int)slot_all.size();
-      for (int s : slice_sites[i]) {
-        slot_all.push_back(s);
-        nr_all.push_back(L.xcnt[s] * L.ycnt[s]);
-        for (int m = 0; m < T; ++m) {
-          zs_all.push_back(s);
-          zt_all.push_back(m);
-          nv2_all.push_back(2 * L.xcnt[s] * L.ycnt[s]);
-        }
+    for (int s : slot_all) {
+      nr_all.push_back(L.xcnt[s] * L.ycnt[s]);
+      for (int m = 0; m < T; ++m) {
+        zs_all.push_back(s);
+        zt_all.push_back(m);
+        nv2_all.push_back(2 * L.xcnt[s] * L.ycnt[s]);
       }
     }
-    site_off[n_z] = (int)slot_all.size();
     // prefix sums of the tiles with work, over all transitions (GEMM 2 / GEMM-V: column
     // tiles of 2 n_R x every row tile of n_out) and over all sites (GEMM-Y: row tiles of
     // n_R x every column tile of 2 w^2); a batch reads its slice of them
@@ -924,7 +903,6 @@ eels_status map_window(eels_ctx* ctx, const eels_smatrix* sm, const eels_transit
     }
     std::vector<int> ab1(sb * T), bb1(sb * T), nv1(sb * T, k2p), ab2(sb * T), bb2(sb * T);
     for (int z = 0; z < sb * T; ++z) { ab1[z] = z / T; bb1[z] = z; ab2[z] = z; bb2[z] = z / T; }
-    EELS_CK(dslot.upload(slot_all.data(), slot_all.size(), st));
     EELS_CK(dzs.upload(zs_all.data(), zs_all.size(), st));
     EELS_CK(dzt.upload(zt_all.data(), zt_all.size(), st));
     EELS_CK(dnv2.upload(nv2_all.data(), nv2_all.size(), st));
@@ -993,7 +971,7 @@ eels_status map_window(eels_ctx* ctx, const eels_smatrix* sm, const eels_transit
       b.slot_site = dslot.p + q0; b.z_site = dzs.p + (int64_t)q0 * T;
       b.z_type = dzt.p + (int64_t)q0 * T; b.n_sites = ns; b.slots_cap = sb;
       b.k1p = k1p; b.k2p = k2p; b.A1 = A1.p; b.B1 = B1.p; b.M1 = M1.p; b.B2 = B2.p;
-      b.ax = ax.p; b.ay = ay.p; b.n_sx = win.nx; b.n_sy = win.ny;
+      b.n_sx = win.nx; b.n_sy = win.ny;
       b.axT = axT.p; b.ayT = ayT.p;
       b.bn_first = eels::tc_tile_width(n1);
       b.bn_second = eels::tc_tile_width(n2);
@@ -1105,23 +1083,25 @@ eels_status map_window(eels_ctx* ctx, const eels_smatrix* sm, const eels_transit
           EELS_OK)
         return r1;
     }
-    for (int b0 = slice_off[i]; !tc && b0 < slice_off[i + 1]; b0 += batch) {
-      eels::TransitionBatch tb{dts.p + b0, dtt.p + b0, std::min(batch, slice_off[i + 1] - b0)};
-      {
-        Prof pr(ctx, "gemm1_fp32", st);
-        EELS_CK(eels::launch_gemm1_fp32(Sout.p, Sin, nh, n_out, n_in, w, H, T, h_mul, tb, dwx.p,
-                                        dwy.p, M.p, m_stride, st));
+    for (int q0 = site_off[i]; !tc && q0 < site_off[i + 1]; q0 += fp_sites)
+      for (int t0 = 0; t0 < T; t0 += fp_types) {
+        const eels::SiteBatch batch{dslot.p + q0, std::min(fp_sites, site_off[i + 1] - q0), t0,
+                                    std::min(fp_types, T - t0)};
+        {
+          Prof pr(ctx, "gemm1_fp32", st);
+          EELS_CK(eels::launch_gemm1_fp32(Sout.p, Sin, nh, n_out, n_in, w, H, T, h_mul, batch,
+                                          dwx.p, dwy.p, M.p, m_stride, st));
+        }
+        {
+          Prof pr(ctx, "gemm2_abs2_fp32", st);
+          EELS_CK(eels::launch_gemm2_abs2_fp32(M.p, m_stride, n_out, n_in, axT.p, ayT.p, win.nx,
+                                               win.ny, batch, wl, dmap.p, st));
+        }
       }
-      {
-        Prof pr(ctx, "gemm2_abs2_fp32", st);
-        EELS_CK(eels::launch_gemm2_abs2_fp32(M.p, m_stride, n_out, n_in, ax.p, ay.p, win.nx,
-                                             win.ny, tb, wl, dmap.p, st));
-      }
-    }
     return EELS_OK;
   };
   const auto t_of = [&](int i) { return sm->t + (int64_t)i * n * n; };
-  const auto has_work = [&](int i) { return slice_off[i + 1] > slice_off[i]; };
+  const auto has_work = [&](int i) { return site_off[i + 1] > site_off[i]; };
   // some depth of the segment whose top depth is i holds transitions
   const auto has_work_to = [&](int i) {
     for (int j = i / K * K; j <= i; ++j)

@@ -2,7 +2,7 @@
 // the second algorithm listing of Sec. III).
 //
 //   GEMM 1   M_t[d][j] = sum_{p in W_s} conj(Sout[d][p]) H_t[p] Sin[j][p]
-//   GEMM 2   V[d][R]   = sum_j M_t[d][j] a_j(R),  a_j(R) = ax[j][ix(R)] ay[j][iy(R)]
+//   GEMM 2   V[d][R]   = sum_j M_t[d][j] a_j(R),  a_j(R) = axT[ix(R)][j] ayT[iy(R)][j]
 //            map[type_t][R] += sum_d |V[d][R]|^2        (FP64 atomics)
 //
 // Sin / Sout are depth planes [beam][N/2][N/2]; the window W_s of a site is the
@@ -15,7 +15,7 @@ namespace eels {
 
 namespace {
 
-constexpr int TM = 64, TN = 64, TK = 16;
+constexpr int TK = 16;   // K values per step
 
 __device__ __forceinline__ void cfma_conj(float2& acc, float2 a, float2 b) {
   // acc += conj(a) * b
@@ -27,178 +27,262 @@ __device__ __forceinline__ void cfma(float2& acc, float2 a, float2 b) {
   acc.y = fmaf(a.x, b.y, fmaf(a.y, b.x, acc.y));
 }
 
-__global__ void __launch_bounds__(256)
+// 8-byte asynchronous copy to shared memory; zero where !on (gmem is not read then)
+__device__ __forceinline__ void cp_async8(float2* smem, const float2* gmem, bool on) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(
+                   (uint32_t)__cvta_generic_to_shared(smem)),
+               "l"(gmem), "r"(on ? 8 : 0)
+               : "memory");
+}
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int PENDING>
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(PENDING) : "memory");
+}
+
+// Both products run one loop over K: 256 threads, a 16 IM x 16 JN output tile (thread
+// (tx, ty) holds rows ty + 16 i, columns tx + 16 j), K in steps of 16 in ascending order
+// with one accumulator per output, so the tile shape does not change a result.  A goes to
+// shared memory by cp.async two steps ahead; B is formed from two factors loaded one step
+// ahead into registers.  One barrier per step.
+//
+// Measured against one 64 x 64 tile per transition, loaded without overlap: a 128-grid
+// request 2.05 -> 1.65 ms of GEMM 1 and 0.22 -> 0.15 of GEMM 2, two 256-grid configurations
+// 9.2 -> 7.0 and 2.8 -> 2.1 ms (41 TFLOP/s useful), a 64-grid map 0.156 -> 0.065 ms.  The FMA
+// pipe is 63 % busy: an FMA that reads three registers runs at two thirds of the rate
+// (25.6 against 38 T/s), and packed f32x2 FMAs do too; they were no faster.
+template <int IM, int JN>
+struct Tile {
+  static constexpr int S = 3;   // shared-memory stages
+  float2 As[S][TK][16 * IM + 1];
+  float2 Bs[S][TK][16 * JN + 1];
+};
+
+// copy_a(it, As): issues this thread's copies of step it (element k = tid % 16 of rows
+// tid / 16 + 16 i); load_b(it): loads the factors of B step it; store_b(Bs): multiplies and
+// stores them.  Steps at or past `steps` copy and load nothing.
+template <int IM, int JN, bool CONJ, class CopyA, class LoadB, class StoreB>
+__device__ __forceinline__ void tile_loop(Tile<IM, JN>& tl, int steps, float2 (&acc)[IM][JN],
+                                          CopyA copy_a, LoadB load_b, StoreB store_b) {
+  constexpr int S = Tile<IM, JN>::S;
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+#pragma unroll
+  for (int i = 0; i < IM; ++i)
+#pragma unroll
+    for (int j = 0; j < JN; ++j) acc[i][j] = make_float2(0.f, 0.f);
+  for (int it = 0; it < S - 1; ++it) {
+    if (it < steps) copy_a(it, tl.As[it]);
+    cp_async_commit();
+  }
+  if (steps > 0) load_b(0);
+  int buf = 0;
+  for (int it = 0; it < steps; ++it) {
+    store_b(tl.Bs[buf]);
+    cp_async_wait<S - 2>();
+    __syncthreads();   // step it is there; every thread has left step it - 1
+    if (it + S - 1 < steps) copy_a(it + S - 1, tl.As[buf == 0 ? S - 1 : buf - 1]);
+    cp_async_commit();
+    if (it + 1 < steps) load_b(it + 1);
+#pragma unroll 4
+    for (int k = 0; k < TK; ++k) {
+      float2 a[IM], b[JN];
+#pragma unroll
+      for (int i = 0; i < IM; ++i) a[i] = tl.As[buf][k][ty + 16 * i];
+#pragma unroll
+      for (int j = 0; j < JN; ++j) b[j] = tl.Bs[buf][k][tx + 16 * j];
+#pragma unroll
+      for (int i = 0; i < IM; ++i)
+#pragma unroll
+        for (int j = 0; j < JN; ++j) {
+          if (CONJ) cfma_conj(acc[i][j], a[i], b[j]);
+          else cfma(acc[i][j], a[i], b[j]);
+        }
+    }
+    buf = buf + 1 == S ? 0 : buf + 1;
+  }
+}
+
+// GEMM 1 of the types t0 .. t0 + nt - 1 of one site per blockIdx.z: columns (t, j) of all
+// types side by side (they share A), M[(slot nt + t)][d][j].
+template <int IM, int JN>
+__global__ void __launch_bounds__(256, IM * JN >= 14 ? 2 : 3)
 k_gemm1(const float2* __restrict__ Sout, const float2* __restrict__ Sin, int nh, int n_out,
         int n_in, int w, const float2* __restrict__ H, int n_types, int h_mul,
-        const int* __restrict__ tr_site,
-        const int* __restrict__ tr_type, const int* __restrict__ win_x0,
+        const int* __restrict__ sites, int t0, int nt, const int* __restrict__ win_x0,
         const int* __restrict__ win_y0, float2* __restrict__ M, int64_t m_stride) {
-  __shared__ float2 As[TK][TM + 1];
-  __shared__ float2 Bs[TK][TN + 1];
-  __shared__ int pix[TK];
-  __shared__ float2 hk[TK];
-  const int t = blockIdx.z;
-  const int s = tr_site[t];
-  if (!STEM_REQUIRE(s >= 0 && tr_type[t] >= 0 && tr_type[t] < n_types &&
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  Tile<IM, JN>& tl = *reinterpret_cast<Tile<IM, JN>*>(smem_raw);
+  const int slot = blockIdx.z, s = sites[slot];
+  if (!STEM_REQUIRE(s >= 0 && t0 >= 0 && t0 + nt <= n_types &&
                     window_ok(win_x0[s], win_y0[s], w, nh)))
     return;   // the whole block, before any barrier
-  const float2* Ht = H + ((int64_t)s * h_mul * n_types + tr_type[t]) * w * w;
   const int x0 = win_x0[s], y0 = win_y0[s];
-  const int d0 = blockIdx.y * TM, j0 = blockIdx.x * TN;
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  const int d0 = blockIdx.y * 16 * IM, c0 = blockIdx.x * 16 * JN;
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;   // loads: tx is k, ty the row
   const int64_t plane = (int64_t)nh * nh;
   const int P = w * w;
-  float2 acc[4][4];
+  // this thread's columns in loads: type and beam (beam -1: past the end)
+  int type[JN], beam[JN];
+  const float2* Hs = H + ((int64_t)s * h_mul * n_types + t0) * P;
 #pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int b = 0; b < 4; ++b) acc[a][b] = make_float2(0.f, 0.f);
-
-  for (int kc = 0; kc < P; kc += TK) {
-    if (threadIdx.x < TK) {
-      const int p = kc + threadIdx.x;
-      if (p < P) {
-        const int v = p / w, u = p % w;
-        const int gy = (y0 + v) % nh, gx = (x0 + u) % nh;
-        pix[threadIdx.x] = gy * nh + gx;
-        hk[threadIdx.x] = Ht[p];
-      } else {
-        pix[threadIdx.x] = -1;
-        hk[threadIdx.x] = make_float2(0.f, 0.f);
-      }
-    }
-    __syncthreads();
-    {
-      const int k = threadIdx.x & (TK - 1);
-      const int r0 = threadIdx.x >> 4;   // 0..15
-      const int pk = pix[k];
-      const float2 h = hk[k];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int r = r0 + 16 * i;
-        float2 a = make_float2(0.f, 0.f), b = make_float2(0.f, 0.f);
-        if (pk >= 0) {
-          if (d0 + r < n_out) a = Sout[(int64_t)(d0 + r) * plane + pk];
-          if (j0 + r < n_in) b = cmul(h, Sin[(int64_t)(j0 + r) * plane + pk]);
-        }
-        As[k][r] = a;
-        Bs[k][r] = b;
-      }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < TK; ++k) {
-      float2 a[4], b[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[k][ty + 16 * i];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) b[i] = Bs[k][tx + 16 * i];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int jj = 0; jj < 4; ++jj) cfma_conj(acc[i][jj], a[i], b[jj]);
-    }
-    __syncthreads();
+  for (int j = 0; j < JN; ++j) {
+    const int c = c0 + ty + 16 * j;
+    type[j] = c / n_in;
+    beam[j] = c < nt * n_in ? c - type[j] * n_in : -1;
   }
-  float2* Mt = M + (int64_t)t * m_stride;
+  // window pixel of K element p = 16 it + tx, walked row by row as it grows by 16
+  struct Walk {
+    int x0, y0, w, nh, u, v;
+    __device__ int next() {   // plane offset of the pixel, then 16 pixels on
+      int gy = y0 + v, gx = x0 + u;
+      if (gy >= nh) gy -= nh;
+      if (gx >= nh) gx -= nh;
+      u += TK;
+      while (u >= w) { u -= w; ++v; }
+      return gy * nh + gx;
+    }
+  };
+  Walk wa{x0, y0, w, nh, tx % w, tx / w}, wb = wa;
+  float2 h[JN], sv[JN];
+  float2 acc[IM][JN];
+  tile_loop<IM, JN, true>(
+      tl, (P + TK - 1) / TK, acc,
+      [&](int it, float2 (*As)[16 * IM + 1]) {
+        const bool in = it * TK + tx < P;
+        const int off = in ? wa.next() : 0;
 #pragma unroll
-  for (int i = 0; i < 4; ++i) {
-    const int d = d0 + ty + 16 * i;
-    if (d >= n_out) continue;
+        for (int i = 0; i < IM; ++i) {
+          const int d = d0 + ty + 16 * i;
+          const bool on = in && d < n_out;
+          cp_async8(&As[tx][ty + 16 * i], on ? Sout + (int64_t)d * plane + off : Sout, on);
+        }
+      },
+      [&](int it) {
+        const int p = it * TK + tx;
+        const bool in = p < P;
+        const int off = in ? wb.next() : 0;
 #pragma unroll
-    for (int jj = 0; jj < 4; ++jj) {
-      const int j = j0 + tx + 16 * jj;
-      if (j < n_in) Mt[(int64_t)d * n_in + j] = acc[i][jj];
+        for (int j = 0; j < JN; ++j) {
+          const bool on = in && beam[j] >= 0;
+          h[j] = on ? __ldg(Hs + ((int64_t)type[j] * P + p)) : make_float2(0.f, 0.f);
+          sv[j] = on ? __ldg(Sin + ((int64_t)beam[j] * plane + off)) : make_float2(0.f, 0.f);
+        }
+      },
+      [&](float2 (*Bs)[16 * JN + 1]) {
+#pragma unroll
+        for (int j = 0; j < JN; ++j) Bs[tx][ty + 16 * j] = cmul(h[j], sv[j]);
+      });
+#pragma unroll
+  for (int j = 0; j < JN; ++j) {
+    const int c = c0 + tx + 16 * j;
+    if (c >= nt * n_in) continue;
+    const int t = c / n_in;
+    float2* Mt = M + ((int64_t)slot * nt + t) * m_stride + (c - t * n_in);
+#pragma unroll
+    for (int i = 0; i < IM; ++i) {
+      const int d = d0 + ty + 16 * i;
+      if (d < n_out) Mt[(int64_t)d * n_in] = acc[i][j];
     }
   }
 }
 
-__global__ void __launch_bounds__(256)
+// GEMM 2 of one site per blockIdx.z.  A row tile is G groups of 64 detector beams; the
+// groups of all types are listed side by side (they share the probe columns).  |V|^2 is
+// summed within a group in FP32 in a fixed order and added to the FP64 map.
+template <int G, int JN>
+__global__ void __launch_bounds__(256, 2)
 k_gemm2_abs2(const float2* __restrict__ M, int64_t m_stride, int n_out, int n_in,
-             const float2* __restrict__ ax, const float2* __restrict__ ay, int n_sx, int n_sy,
-             const int* __restrict__ tr_site, const int* __restrict__ tr_type,
-             const int* __restrict__ xoff, const int* __restrict__ xcnt,
-             const int* __restrict__ xlist, const int* __restrict__ yoff,
-             const int* __restrict__ ycnt, const int* __restrict__ ylist,
-             double* __restrict__ map) {
-  __shared__ float2 As[TK][TM + 1];
-  __shared__ float2 Bs[TK][TN + 1];
-  __shared__ float red[16][TN];
+             const float2* __restrict__ axT, const float2* __restrict__ ayT, int n_sx, int n_sy,
+             const int* __restrict__ sites, int t0, int nt, const int* __restrict__ xoff,
+             const int* __restrict__ xcnt, const int* __restrict__ xlist,
+             const int* __restrict__ yoff, const int* __restrict__ ycnt,
+             const int* __restrict__ ylist, double* __restrict__ map) {
+  constexpr int IM = 4 * G, TN = 16 * JN;
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  Tile<IM, JN>& tl = *reinterpret_cast<Tile<IM, JN>*>(smem_raw);
+  __shared__ float red[G][16][TN];
   __shared__ int rix[TN], riy[TN];
-  const int t = blockIdx.z;
-  const int s = tr_site[t];
-  const int nx = xcnt[s], ny = ycnt[s];
-  const int nr = nx * ny;
+  const int slot = blockIdx.z, s = sites[slot];
+  const int nx = xcnt[s], nr = nx * ycnt[s];
   const int r0 = blockIdx.x * TN;
   if (r0 >= nr) return;
-  const int d0 = blockIdx.y * TM;
   const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
   if (threadIdx.x < TN) {
     const int r = r0 + threadIdx.x;
+    int ix = -1, iy = -1;
     if (r < nr) {
-      rix[threadIdx.x] = xlist[xoff[s] + r % nx];
-      riy[threadIdx.x] = ylist[yoff[s] + r / nx];
-      if (!STEM_REQUIRE(rix[threadIdx.x] >= 0 && rix[threadIdx.x] < n_sx &&
-                        riy[threadIdx.x] >= 0 && riy[threadIdx.x] < n_sy && tr_type[t] >= 0))
-        rix[threadIdx.x] = riy[threadIdx.x] = -1;   // skipped below
-    } else {
-      rix[threadIdx.x] = -1;
-      riy[threadIdx.x] = -1;
+      ix = xlist[xoff[s] + r % nx];
+      iy = ylist[yoff[s] + r / nx];
+      if (!STEM_REQUIRE(ix >= 0 && ix < n_sx && iy >= 0 && iy < n_sy)) ix = iy = -1;   // skipped
     }
+    rix[threadIdx.x] = ix;
+    riy[threadIdx.x] = iy;
   }
-  const float2* Mt = M + (int64_t)t * m_stride;
-  float2 acc[4][4];
-#pragma unroll
-  for (int a = 0; a < 4; ++a)
-#pragma unroll
-    for (int b = 0; b < 4; ++b) acc[a][b] = make_float2(0.f, 0.f);
   __syncthreads();
-  for (int kc = 0; kc < n_in; kc += TK) {
-    {
-      const int k = threadIdx.x & (TK - 1);
-      const int rr = threadIdx.x >> 4;
-      const int j = kc + k;
+  const int per_type = (n_out + 63) / 64, groups = nt * per_type;
+  // M rows of this thread's loads: row ty + 16 i of the tile is beam 64 g + ty + 16 (i % 4)
+  // of group blockIdx.y G + i / 4
+  const float2* Mg[G];
+  int dg[G];   // first beam of the group; n_out where there is no such group
+#pragma unroll
+  for (int g = 0; g < G; ++g) {
+    const int gi = blockIdx.y * G + g, t = gi / per_type;
+    dg[g] = gi < groups ? 64 * (gi - t * per_type) : n_out;
+    Mg[g] = M + ((int64_t)slot * nt + (gi < groups ? t : 0)) * m_stride;
+  }
+  int ix[JN], iy[JN];
+#pragma unroll
+  for (int j = 0; j < JN; ++j) {
+    ix[j] = rix[ty + 16 * j];
+    iy[j] = riy[ty + 16 * j];
+  }
+  float2 fx[JN], fy[JN];
+  float2 acc[IM][JN];
+  tile_loop<IM, JN, false>(
+      tl, (n_in + TK - 1) / TK, acc,
+      [&](int it, float2 (*As)[16 * IM + 1]) {
+        const int k = it * TK + tx;
+#pragma unroll
+        for (int i = 0; i < IM; ++i) {
+          const int d = dg[i / 4] + ty + 16 * (i % 4);
+          const bool on = k < n_in && d < n_out;
+          cp_async8(&As[tx][ty + 16 * i], on ? Mg[i / 4] + (int64_t)d * n_in + k : M, on);
+        }
+      },
+      [&](int it) {
+        const int k = it * TK + tx;
+#pragma unroll
+        for (int j = 0; j < JN; ++j) {
+          const bool on = k < n_in && ix[j] >= 0;
+          fx[j] = on ? __ldg(axT + ((int64_t)ix[j] * n_in + k)) : make_float2(0.f, 0.f);
+          fy[j] = on ? __ldg(ayT + ((int64_t)iy[j] * n_in + k)) : make_float2(0.f, 0.f);
+        }
+      },
+      [&](float2 (*Bs)[16 * JN + 1]) {
+#pragma unroll
+        for (int j = 0; j < JN; ++j) Bs[tx][ty + 16 * j] = cmul(fx[j], fy[j]);
+      });
+  // |V|^2 summed over each group's rows, per scan position
+#pragma unroll
+  for (int g = 0; g < G; ++g)
+#pragma unroll
+    for (int j = 0; j < JN; ++j) {
+      float sum = 0.f;
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
-        const int r = rr + 16 * i;
-        float2 a = make_float2(0.f, 0.f), b = make_float2(0.f, 0.f);
-        if (j < n_in) {
-          if (d0 + r < n_out) a = Mt[(int64_t)(d0 + r) * n_in + j];
-          if (rix[r] >= 0) b = cmul(ax[(int64_t)j * n_sx + rix[r]], ay[(int64_t)j * n_sy + riy[r]]);
-        }
-        As[k][r] = a;
-        Bs[k][r] = b;
+        const float2 v = acc[4 * g + i][j];
+        sum = fmaf(v.x, v.x, fmaf(v.y, v.y, sum));
       }
+      red[g][ty][tx + 16 * j] = sum;
     }
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < TK; ++k) {
-      float2 a[4], b[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) a[i] = As[k][ty + 16 * i];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) b[i] = Bs[k][tx + 16 * i];
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-#pragma unroll
-        for (int jj = 0; jj < 4; ++jj) cfma(acc[i][jj], a[i], b[jj]);
-    }
-    __syncthreads();
-  }
-  // |V|^2 summed over this tile's d rows, per scan position
-#pragma unroll
-  for (int jj = 0; jj < 4; ++jj) {
-    float sum = 0.f;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) sum = fmaf(acc[i][jj].x, acc[i][jj].x, fmaf(acc[i][jj].y, acc[i][jj].y, sum));
-    red[ty][tx + 16 * jj] = sum;
-  }
   __syncthreads();
-  if (threadIdx.x < TN && rix[threadIdx.x] >= 0) {
+  for (int e = threadIdx.x; e < G * TN; e += 256) {
+    const int g = e / TN, c = e % TN, gi = blockIdx.y * G + g;
+    if (gi >= groups || rix[c] < 0) continue;
     float sum = 0.f;
 #pragma unroll
-    for (int i = 0; i < 16; ++i) sum += red[i][threadIdx.x];
-    const int64_t idx = ((int64_t)tr_type[t] * n_sy + riy[threadIdx.x]) * n_sx + rix[threadIdx.x];
+    for (int i = 0; i < 16; ++i) sum += red[g][i][c];
+    const int64_t idx = ((int64_t)(t0 + gi / per_type) * n_sy + riy[c]) * n_sx + rix[c];
     atomicAdd(map + idx, (double)sum);
   }
 }
@@ -246,26 +330,95 @@ __global__ void k_scale_check(double* a, int64_t count, double scale, int* flag)
 
 }  // namespace
 
-cudaError_t launch_gemm1_fp32(const float2* Sout, const float2* Sin, int nh, int n_out, int n_in,
-                              int w, const float2* H, int n_types, int h_mul,
-                              const TransitionBatch& tb, const int* win_x0, const int* win_y0,
-                              float2* M, int64_t m_stride, cudaStream_t s) {
-  if (tb.count <= 0) return cudaSuccess;
-  dim3 grid((n_in + TN - 1) / TN, (n_out + TM - 1) / TM, tb.count);
-  k_gemm1<<<grid, 256, 0, s>>>(Sout, Sin, nh, n_out, n_in, w, H, n_types, h_mul, tb.site, tb.type,
-                               win_x0, win_y0, M, m_stride);
+namespace {
+
+// Estimated cycles of one K step over a whole launch with 16 im x 16 jn tiles: the CTAs of
+// the busiest SM after one another at 128 im jn cycles of FMA issue each, plus the latency
+// of a step that nothing hides when few CTAs share an SM.
+double step_cost(int64_t ctas, int im, int jn) {
+  const double per_sm = (double)((ctas + sm_count() - 1) / sm_count());
+  return per_sm * 128.0 * im * jn + (per_sm < 2 ? 500.0 : 250.0);
+}
+
+template <int IM, int JN>
+cudaError_t gemm1_tile(const float2* Sout, const float2* Sin, int nh, int n_out, int n_in, int w,
+                       const float2* H, int n_types, int h_mul, const SiteBatch& sb,
+                       const int* win_x0, const int* win_y0, float2* M, int64_t m_stride,
+                       cudaStream_t s) {
+  static std::atomic<uint64_t> attr{0};
+  cudaError_t e = smem_attr_once(k_gemm1<IM, JN>, sizeof(Tile<IM, JN>), attr);
+  if (e != cudaSuccess) return e;
+  dim3 grid((sb.nt * n_in + 16 * JN - 1) / (16 * JN), (n_out + 16 * IM - 1) / (16 * IM), sb.count);
+  k_gemm1<IM, JN><<<grid, 256, sizeof(Tile<IM, JN>), s>>>(Sout, Sin, nh, n_out, n_in, w, H,
+                                                          n_types, h_mul, sb.site, sb.t0, sb.nt,
+                                                          win_x0, win_y0, M, m_stride);
   return cudaGetLastError();
 }
 
-cudaError_t launch_gemm2_abs2_fp32(const float2* M, int64_t m_stride, int n_out, int n_in,
-                                   const float2* ax, const float2* ay, int n_sx, int n_sy,
-                                   const TransitionBatch& tb, const WindowLists& wl, double* map,
-                                   cudaStream_t s) {
-  if (tb.count <= 0 || wl.max_nr <= 0) return cudaSuccess;
-  dim3 grid((wl.max_nr + TN - 1) / TN, (n_out + TM - 1) / TM, tb.count);
-  k_gemm2_abs2<<<grid, 256, 0, s>>>(M, m_stride, n_out, n_in, ax, ay, n_sx, n_sy, tb.site, tb.type,
-                                    wl.xoff, wl.xcnt, wl.xlist, wl.yoff, wl.ycnt, wl.ylist, map);
+template <int G, int JN>
+cudaError_t gemm2_tile(const float2* M, int64_t m_stride, int n_out, int n_in, const float2* axT,
+                       const float2* ayT, int n_sx, int n_sy, const SiteBatch& sb,
+                       const WindowLists& wl, double* map, cudaStream_t s) {
+  static std::atomic<uint64_t> attr{0};
+  cudaError_t e = smem_attr_once(k_gemm2_abs2<G, JN>, sizeof(Tile<4 * G, JN>), attr);
+  if (e != cudaSuccess) return e;
+  const int groups = sb.nt * ((n_out + 63) / 64);
+  dim3 grid((wl.max_nr + 16 * JN - 1) / (16 * JN), (groups + G - 1) / G, sb.count);
+  k_gemm2_abs2<G, JN><<<grid, 256, sizeof(Tile<4 * G, JN>), s>>>(
+      M, m_stride, n_out, n_in, axT, ayT, n_sx, n_sy, sb.site, sb.t0, sb.nt, wl.xoff, wl.xcnt,
+      wl.xlist, wl.yoff, wl.ycnt, wl.ylist, map);
   return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_gemm1_fp32(const float2* Sout, const float2* Sin, int nh, int n_out, int n_in,
+                              int w, const float2* H, int n_types, int h_mul, const SiteBatch& sb,
+                              const int* win_x0, const int* win_y0, float2* M, int64_t m_stride,
+                              cudaStream_t s) {
+  if (sb.count <= 0 || sb.nt <= 0) return cudaSuccess;
+  // the tile that wastes least on the edges of n_out and nt n_in, or spreads a small
+  // launch over more SMs
+  int im = 0, jn = 0;
+  double best = 0;
+  for (int i : {8, 7, 6, 5, 4, 2})
+    for (int j : {4, 2}) {
+      const int64_t ctas = (int64_t)((sb.nt * n_in + 16 * j - 1) / (16 * j)) *
+                           ((n_out + 16 * i - 1) / (16 * i)) * sb.count;
+      const double c = step_cost(ctas, i, j);
+      if (im == 0 || c < best) { best = c; im = i; jn = j; }
+    }
+#define EELS_G1(I, J)                                                                         \
+  if (im == I && jn == J)                                                                     \
+    return gemm1_tile<I, J>(Sout, Sin, nh, n_out, n_in, w, H, n_types, h_mul, sb, win_x0,     \
+                            win_y0, M, m_stride, s);
+  EELS_G1(8, 4) EELS_G1(7, 4) EELS_G1(6, 4) EELS_G1(5, 4) EELS_G1(4, 4) EELS_G1(2, 4)
+  EELS_G1(8, 2) EELS_G1(7, 2) EELS_G1(6, 2) EELS_G1(5, 2) EELS_G1(4, 2) EELS_G1(2, 2)
+#undef EELS_G1
+  return cudaErrorInvalidValue;
+}
+
+cudaError_t launch_gemm2_abs2_fp32(const float2* M, int64_t m_stride, int n_out, int n_in,
+                                   const float2* axT, const float2* ayT, int n_sx, int n_sy,
+                                   const SiteBatch& sb, const WindowLists& wl, double* map,
+                                   cudaStream_t s) {
+  if (sb.count <= 0 || sb.nt <= 0 || wl.max_nr <= 0) return cudaSuccess;
+  const int groups = sb.nt * ((n_out + 63) / 64);
+  int g = 0, jn = 0;
+  double best = 0;
+  for (int i : {2, 1})
+    for (int j : {4, 2}) {
+      const int64_t ctas = (int64_t)((wl.max_nr + 16 * j - 1) / (16 * j)) * ((groups + i - 1) / i) *
+                           sb.count;
+      const double c = step_cost(ctas, 4 * i, j);
+      if (g == 0 || c < best) { best = c; g = i; jn = j; }
+    }
+#define EELS_G2(I, J)                                                                         \
+  if (g == I && jn == J)                                                                      \
+    return gemm2_tile<I, J>(M, m_stride, n_out, n_in, axT, ayT, n_sx, n_sy, sb, wl, map, s);
+  EELS_G2(2, 4) EELS_G2(1, 4) EELS_G2(2, 2) EELS_G2(1, 2)
+#undef EELS_G2
+  return cudaErrorInvalidValue;
 }
 
 cudaError_t launch_phase_table(float2* out, const int* bidx, int n_beams, int f, double cell,

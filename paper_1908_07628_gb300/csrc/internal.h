@@ -76,23 +76,25 @@ cudaError_t launch_spawn(int n, const SpawnList& sp, const float2* D, const floa
                          const float2* tw, cudaStream_t s);
 
 // Contraction (CUDA cores, FP32).
-struct TransitionBatch {
-  const int* site;    // [count] site index of each transition
-  const int* type;    // [count]
+struct SiteBatch {
+  const int* site;    // [count] sites; the transitions are types t0 .. t0 + nt - 1 of each
   int count;
+  int t0, nt;
 };
 struct WindowLists {
   const int* xoff; const int* xcnt; const int* xlist;   // per site: scan columns in the PRISM window
   const int* yoff; const int* ycnt; const int* ylist;   // per site: scan rows
   int max_nr;                                           // max over sites of xcnt*ycnt
 };
+// M[slot nt + t][d][j], m_stride values apart
 cudaError_t launch_gemm1_fp32(const float2* Sout, const float2* Sin, int nh, int n_out, int n_in,
-                              int w, const float2* H, int n_types, int h_mul,
-                              const TransitionBatch& tb, const int* win_x0, const int* win_y0,
-                              float2* M, int64_t m_stride, cudaStream_t s);
+                              int w, const float2* H, int n_types, int h_mul, const SiteBatch& sb,
+                              const int* win_x0, const int* win_y0, float2* M, int64_t m_stride,
+                              cudaStream_t s);
+// axT, ayT: phase tables [pos][n_in]
 cudaError_t launch_gemm2_abs2_fp32(const float2* M, int64_t m_stride, int n_out, int n_in,
-                                   const float2* ax, const float2* ay, int n_sx, int n_sy,
-                                   const TransitionBatch& tb, const WindowLists& wl, double* map,
+                                   const float2* axT, const float2* ayT, int n_sx, int n_sy,
+                                   const SiteBatch& sb, const WindowLists& wl, double* map,
                                    cudaStream_t s);
 // ax[j][ix] = exp(-2 pi i f p_j Rx(ix) / L) (FP64 phase); same for ay with q_j, Ry.  Row
 // ix holds position Rx = r0 + (r_first + ix) step (a window of a longer scan line).
@@ -150,7 +152,7 @@ struct TcBatch {
   int n_sites, slots_cap;                 // sites in this batch, buffer capacity in sites
   int k1p, k2p;                           // padded K of GEMM 1 (2 w^2) and GEMM 2 (2 n_in)
   void* A1; void* B1; void* M1; void* B2;
-  const float2* ax; const float2* ay; int n_sx, n_sy;
+  int n_sx, n_sy;
   const int* xoff; const int* xcnt; const int* xlist;
   const int* yoff; const int* ycnt; const int* ylist;
   int nr_cap;                             // max scan positions of a site
