@@ -1385,17 +1385,23 @@ eels_status eels_elastic_images(eels_ctx* ctx, const eels_smatrix* sm, const eel
   if (r != EELS_OK) return r;
   DevBuf<int> dwx, dwy, dbp, dbq;
   DevBuf<uint8_t> dmask;
-  DevBuf<float2> ax, ay, cuts;
+  DevBuf<float2> axT, ayT, cuts;
   DevBuf<double> dimg;
   EELS_CK(dwx.upload(wx.data(), wx.size(), st));
   EELS_CK(dwy.upload(wy.data(), wy.size(), st));
   EELS_CK(dmask.upload(mask.data(), mask.size(), st));
   EELS_CK(dbp.upload(sm->bp.data(), n_in, st));
   EELS_CK(dbq.upload(sm->bq.data(), n_in, st));
-  EELS_CK(ax.alloc((size_t)n_in * sc->n_sx, st));
-  EELS_CK(ay.alloc((size_t)n_in * sc->n_sy, st));
-  EELS_CK(eels::launch_phase_table(ax.p, dbp.p, n_in, f, sm->cell, sc->x0, sc->step_x, sc->n_sx, st));
-  EELS_CK(eels::launch_phase_table(ay.p, dbq.p, n_in, f, sm->cell, sc->y0, sc->step_y, sc->n_sy, st));
+  EELS_CK(axT.alloc((size_t)n_in * sc->n_sx, st));
+  EELS_CK(ayT.alloc((size_t)n_in * sc->n_sy, st));
+  EELS_CK(eels::launch_phase_table(axT.p, dbp.p, n_in, f, sm->cell, sc->x0, sc->step_x, sc->n_sx,
+                                   st, 1));
+  EELS_CK(eels::launch_phase_table(ayT.p, dbq.p, n_in, f, sm->cell, sc->y0, sc->step_y, sc->n_sy,
+                                   st, 1));
+  int max_span = 0;   // of the column origins of probes that one CTA may take together
+  for (int i = 0; i < sc->n_sx; ++i)
+    for (int k = i; k < std::min(i + eels::kMaxCutProbes, sc->n_sx); ++k)
+      max_span = std::max(max_span, (wx[k] - wx[i] + nh) % nh);
   EELS_CK(dimg.alloc((size_t)n_det * n_img, st));
   EELS_CK(cudaMemsetAsync(dimg.p, 0, sizeof(double) * n_det * n_img, st));
   // scan rows in batches whose cuts fit in ~1 GiB
@@ -1406,8 +1412,8 @@ eels_status eels_elastic_images(eels_ctx* ctx, const eels_smatrix* sm, const eel
     const int nr = std::min(rows_b, sc->n_sy - iy0);
     {
       Prof pr(ctx, "exit_cut", st);
-      EELS_CK(eels::launch_exit_cut(sm->s_exit, n_in, nh, m, ax.p, ay.p, sc->n_sx, sc->n_sy,
-                                    dwx.p, dwy.p, iy0, nr, cuts.p, st));
+      EELS_CK(eels::launch_exit_cut(sm->s_exit, n_in, nh, m, axT.p, ayT.p, sc->n_sx, sc->n_sy,
+                                    dwx.p, dwy.p, iy0, nr, max_span, cuts.p, st));
     }
     Prof pr(ctx, "cut_fft_detect", st);
     EELS_CK(eels::launch_cut_detect(m, cuts.p, nr * sc->n_sx, dmask.p, n_det, sc->n_sx, iy0,

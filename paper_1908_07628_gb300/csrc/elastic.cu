@@ -19,32 +19,60 @@ namespace eels {
 
 namespace {
 
-constexpr int kCutProbes = 16;    // probes of one scan row per CTA of the cut pass
-constexpr int kCutThreads = 256;
+constexpr int kCutWarps = 8;      // warps per CTA of the cut pass
 constexpr int kBeamChunk = 32;    // beams whose coefficients are staged at a time
+constexpr int kBeamAhead = 2;     // beams whose S values a thread loads together; divides kBeamChunk
 constexpr int kFftWarps = 8;
 
-// One CTA: up to 16 consecutive probes ix0.. of scan row iy, one cut row y'.  Every
-// S_exit element of the group's column span is loaded once and used by all probes
-// whose cut contains it.
-__global__ void __launch_bounds__(kCutThreads)
+// Packed pairs of floats: one instruction for the real and imaginary part, each rounded as
+// the scalar operation.
+__device__ __forceinline__ uint64_t pack2(float lo, float hi) {
+  uint64_t d;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
+  return d;
+}
+__device__ __forceinline__ uint64_t add2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ uint64_t fma2(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t d;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+  return d;
+}
+
+// Cut pass.  A CTA takes G consecutive probes ix0 .. of one scan row, a thread one column of
+// two neighbouring cut rows (elements (row pair, column) in one list, so that no lane is
+// left over at the end of a row); every S_exit value of the group's column span is loaded once
+// for all its probes.  Each product is rounded and then added (six FP32 operations per
+// complex product), beams in ascending order.  Bound by the FP32 pipe: coefficients lie in
+// shared memory as (c.x, c.x), (c.y, c.y), so that a product is three packed instructions
+// and half of the issue slots are left for the loads, and two rows share each coefficient.
+// 512-grid crystal, f = 2, 32 x 32 probes, 593 beams: 4.87 -> 2.65 ms (one row per CTA with
+// scalar products before); the FP32 pipe alone would take 1.57 ms for the cuts' own pixels.
+template <int G>
+__global__ void __launch_bounds__(kCutWarps * 32, 2)
 k_exit_cut(const float2* __restrict__ S, int n_in, int nh, int m,
-           const float2* __restrict__ ax, const float2* __restrict__ ay, int n_sx, int n_sy,
+           const float2* __restrict__ axT, const float2* __restrict__ ayT, int n_sx, int n_sy,
            const int* __restrict__ wx, const int* __restrict__ wy, int iy0,
            float2* __restrict__ out) {
-  __shared__ __align__(16) float2 coef[kBeamChunk][kCutProbes];
-  __shared__ int dx[kCutProbes];
-  const int ix0 = blockIdx.x * kCutProbes;
-  const int np = min(kCutProbes, n_sx - ix0);
-  const int yp = blockIdx.y;
+  __shared__ ulonglong2 coef[2][kBeamChunk][G];   // (c.x, c.x), (c.y, c.y)
+  __shared__ int dx[G];
+  const int ix0 = blockIdx.x * G;
+  const int np = min(G, n_sx - ix0);
   const int iyl = blockIdx.z;
   const int iy = iy0 + iyl;
   // window origins on the grid (the block's row origin and first column origin decide
   // for the whole block; a bad later column origin is replaced by the first)
   if (!STEM_REQUIRE(wy[iy] >= 0 && wy[iy] < nh && wx[ix0] >= 0 && wx[ix0] < nh)) return;
-  const int y = (wy[iy] + yp) % nh;
   const int xa = wx[ix0];
-  if (threadIdx.x < kCutProbes) {
+  if (threadIdx.x < G) {
     int xg = threadIdx.x < np ? wx[ix0 + threadIdx.x] : xa;
     if (!STEM_REQUIRE(xg >= 0 && xg < nh)) xg = xa;
     dx[threadIdx.x] = (xg - xa + nh) % nh;
@@ -52,49 +80,82 @@ k_exit_cut(const float2* __restrict__ S, int n_in, int nh, int m,
   __syncthreads();
   int span = 0;
   for (int g = 0; g < np; ++g) span = max(span, dx[g]);
-  const int U = min(span + m, nh);   // columns xa .. xa + U - 1 (cyclic)
+  const int U = min(span + m, nh);          // columns xa .. xa + U - 1 (cyclic)
+  const int first = blockIdx.y * kCutWarps * 32;   // this CTA's (row pair, column) elements
+  if (first >= (m / 2) * U) return;                // the same for the whole block
+  const int yp = 2 * ((first + (int)threadIdx.x) / U), u = (first + (int)threadIdx.x) % U;
+  const bool active = yp < m;
   const int64_t plane = (int64_t)nh * nh;
-  const float2* Srow = S + (int64_t)y * nh;
+  const int x = (xa + (active ? u : 0)) % nh, y0 = (wy[iy] + (active ? yp : 0)) % nh;
+  const int y1 = y0 + 1 == nh ? 0 : y0 + 1;
+  const float2* S0 = S + (int64_t)y0 * nh + x;
+  const int d1 = (y1 - y0) * nh;            // the second row's offset
 
-  for (int u0 = 0; u0 < U; u0 += kCutThreads) {
-    const int u = u0 + threadIdx.x;
-    const bool active = u < U;
-    const int x = (xa + (active ? u : 0)) % nh;
-    float2 acc[kCutProbes];
+  // coefficients of the beams j0 .. j0 + kBeamChunk - 1 (zero past n_in and past the probes)
+  auto stage = [&](int j0, int buf) {
+    for (int idx = threadIdx.x; idx < kBeamChunk * G; idx += kCutWarps * 32) {
+      const int jj = idx % kBeamChunk, g = idx / kBeamChunk, j = j0 + jj;
+      float2 c = make_float2(0.f, 0.f);
+      if (j < n_in && g < np)
+        c = cmul(__ldg(axT + (int64_t)(ix0 + g) * n_in + j), __ldg(ayT + (int64_t)iy * n_in + j));
+      coef[buf][jj][g] = make_ulonglong2(pack2(c.x, c.x), pack2(c.y, c.y));
+    }
+  };
+  uint64_t acc[2][G];
 #pragma unroll
-    for (int g = 0; g < kCutProbes; ++g) acc[g] = make_float2(0.f, 0.f);
-    for (int j0 = 0; j0 < n_in; j0 += kBeamChunk) {
-      const int jc = min(kBeamChunk, n_in - j0);
-      __syncthreads();
-      for (int idx = threadIdx.x; idx < kBeamChunk * kCutProbes; idx += kCutThreads) {
-        const int jj = idx / kCutProbes, g = idx % kCutProbes;
-        float2 c = make_float2(0.f, 0.f);
-        if (jj < jc && g < np)
-          c = cmul(ax[(int64_t)(j0 + jj) * n_sx + ix0 + g], ay[(int64_t)(j0 + jj) * n_sy + iy]);
-        coef[jj][g] = c;
-      }
-      __syncthreads();
-      if (active) {
-        for (int jj = 0; jj < jc; ++jj) {
-          const float2 s = __ldg(Srow + (int64_t)(j0 + jj) * plane + x);
-          const float4* c4 = reinterpret_cast<const float4*>(&coef[jj][0]);
+  for (int g = 0; g < G; ++g) acc[0][g] = acc[1][g] = 0ull;
+  // S values of the beams j .. j + kBeamAhead - 1, loaded while the ones before are used
+  float2 ahead[2][kBeamAhead];
+  auto load = [&](int j) {
 #pragma unroll
-          for (int g2 = 0; g2 < kCutProbes / 2; ++g2) {
-            const float4 c = c4[g2];
-            acc[2 * g2] = cadd(acc[2 * g2], cmul(make_float2(c.x, c.y), s));
-            acc[2 * g2 + 1] = cadd(acc[2 * g2 + 1], cmul(make_float2(c.z, c.w), s));
-          }
+    for (int e = 0; e < kBeamAhead; ++e) {
+      const float2* p = S0 + (int64_t)(j + e) * plane;
+      const bool on = active && j + e < n_in;
+      ahead[0][e] = on ? __ldg(p) : make_float2(0.f, 0.f);
+      ahead[1][e] = on ? __ldg(p + d1) : make_float2(0.f, 0.f);
+    }
+  };
+  stage(0, 0);
+  load(0);
+  int buf = 0;
+  for (int j0 = 0; j0 < n_in; j0 += kBeamChunk, buf ^= 1) {
+    __syncthreads();
+    if (j0 + kBeamChunk < n_in) stage(j0 + kBeamChunk, buf ^ 1);
+    if (!active) continue;
+    const int jc = min(kBeamChunk, n_in - j0);
+    for (int jj = 0; jj < jc; jj += kBeamAhead) {
+      float2 s[2][kBeamAhead];
+#pragma unroll
+      for (int e = 0; e < kBeamAhead; ++e) s[0][e] = ahead[0][e], s[1][e] = ahead[1][e];
+      load(j0 + jj + kBeamAhead);
+#pragma unroll
+      for (int e = 0; e < kBeamAhead; ++e) {
+        if (jj + e >= jc) break;
+        uint64_t v[2], r[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          v[h] = pack2(s[h][e].x, s[h][e].y);
+          r[h] = pack2(-s[h][e].y, s[h][e].x);
+        }
+#pragma unroll
+        for (int g = 0; g < G; ++g) {
+          const ulonglong2 c = coef[buf][jj + e][g];
+#pragma unroll
+          for (int h = 0; h < 2; ++h)
+            acc[h][g] = add2(acc[h][g], fma2(c.x, v[h], mul2(c.y, r[h])));
         }
       }
     }
-    if (active) {
+  }
+  if (active) {
 #pragma unroll
-      for (int g = 0; g < kCutProbes; ++g) {
-        if (g < np) {
-          const int xp = (u - dx[g] + nh) % nh;
-          if (xp < m)
-            out[(((int64_t)iyl * n_sx + ix0 + g) * m + yp) * m + xp] = acc[g];
-        }
+    for (int g = 0; g < G; ++g) {
+      const int xp = (u - dx[g] + nh) % nh;
+      if (g < np && xp < m) {
+        uint64_t* dst = reinterpret_cast<uint64_t*>(
+            out + (((int64_t)iyl * n_sx + ix0 + g) * m + yp) * m + xp);
+        dst[0] = acc[0][g];
+        dst[m] = acc[1][g];
       }
     }
   }
@@ -256,13 +317,34 @@ bool cut_supported(int m) {
   }
 }
 
-cudaError_t launch_exit_cut(const float2* S, int n_in, int nh, int m, const float2* ax,
-                            const float2* ay, int n_sx, int n_sy, const int* wx, const int* wy,
-                            int iy0, int n_rows, float2* out, cudaStream_t s) {
-  if (n_rows <= 0) return cudaSuccess;
-  dim3 g((unsigned)((n_sx + kCutProbes - 1) / kCutProbes), (unsigned)m, (unsigned)n_rows);
-  k_exit_cut<<<g, kCutThreads, 0, s>>>(S, n_in, nh, m, ax, ay, n_sx, n_sy, wx, wy, iy0, out);
+namespace {
+
+template <int G>
+cudaError_t exit_cut_g(const float2* S, int n_in, int nh, int m, const float2* axT,
+                       const float2* ayT, int n_sx, int n_sy, const int* wx, const int* wy,
+                       int iy0, int n_rows, int max_span, float2* out, cudaStream_t s) {
+  const int elements = (m / 2) * std::min(m + max_span, nh), threads = kCutWarps * 32;
+  dim3 g((unsigned)((n_sx + G - 1) / G), (unsigned)((elements + threads - 1) / threads),
+         (unsigned)n_rows);
+  k_exit_cut<G><<<g, kCutWarps * 32, 0, s>>>(S, n_in, nh, m, axT, ayT, n_sx, n_sy, wx, wy, iy0,
+                                             out);
   return cudaGetLastError();
+}
+
+}  // namespace
+
+cudaError_t launch_exit_cut(const float2* S, int n_in, int nh, int m, const float2* axT,
+                            const float2* ayT, int n_sx, int n_sy, const int* wx, const int* wy,
+                            int iy0, int n_rows, int max_span, float2* out, cudaStream_t s) {
+  if (n_rows <= 0) return cudaSuccess;
+  // probes per CTA: 16 share each S value best; fewer where 16 would leave more than a
+  // quarter of the accumulators without a probe
+  const int pad16 = (n_sx + 15) / 16 * 16, pad8 = (n_sx + 7) / 8 * 8;
+  if (n_sx <= 4)
+    return exit_cut_g<4>(S, n_in, nh, m, axT, ayT, n_sx, n_sy, wx, wy, iy0, n_rows, max_span, out, s);
+  if (4 * (pad16 - pad8) > pad16)
+    return exit_cut_g<8>(S, n_in, nh, m, axT, ayT, n_sx, n_sy, wx, wy, iy0, n_rows, max_span, out, s);
+  return exit_cut_g<16>(S, n_in, nh, m, axT, ayT, n_sx, n_sy, wx, wy, iy0, n_rows, max_span, out, s);
 }
 
 cudaError_t launch_cut_detect(int m, float2* X, int n_cut, const uint8_t* mask, int n_det,
