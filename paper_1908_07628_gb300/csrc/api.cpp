@@ -12,6 +12,7 @@
 #include <cstdio>
 #include <cstring>
 #include <map>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -44,7 +45,6 @@ struct eels_ctx {
   struct Choice { int assoc; int narrow1, narrow2; };
   std::map<std::vector<int64_t>, Choice> assoc_cache;
   std::string err;
-  std::map<int, float2*> tw;   // device twiddle table exp(-2 pi i k/N), by N
   // kernel timing records (eels_profile_enable)
   bool profiling = false;
   struct Rec { const char* name; cudaEvent_t a, b; };
@@ -153,6 +153,38 @@ struct DevBuf {
   }
 };
 
+// Device address of an array inside a Pack.
+template <typename T>
+struct PackPtr {
+  T* p = nullptr;
+};
+
+// Small host arrays that a call needs on the device, sent in one buffer by one copy: a map
+// has about thirty of them, and an allocation, a pageable copy and a free for each cost a
+// small map more than its kernels (64 grid: 258 -> 190 us).
+struct Pack {
+  std::vector<unsigned char> host;
+  struct Item { void** at; size_t offset; };
+  std::vector<Item> items;
+  DevBuf<unsigned char> dev;
+  template <typename T>
+  void add(PackPtr<T>& d, const T* src, size_t count) {
+    const size_t offset = (host.size() + 255) / 256 * 256;
+    host.resize(offset + std::max<size_t>(count, 1) * sizeof(T));
+    if (count) std::memcpy(host.data() + offset, src, count * sizeof(T));
+    items.push_back({(void**)&d.p, offset});
+  }
+  template <typename T>
+  void add(PackPtr<T>& d, const std::vector<T>& v) { add(d, v.data(), v.size()); }
+  // one allocation and one copy; the host bytes are staged by the driver before this returns
+  cudaError_t upload(cudaStream_t st) {
+    cudaError_t e = dev.upload(host.data(), host.size(), st);
+    if (e != cudaSuccess) return e;
+    for (const Item& i : items) *i.at = dev.p + i.offset;
+    return cudaSuccess;
+  }
+};
+
 // f-lattice beams (p, q), k = f(p, q)/L, with lambda |k| <= angle (Sec. III).
 void lattice_beams(int n, double cell, double lam, int f, double angle, std::vector<int>& p,
                    std::vector<int>& q) {
@@ -214,9 +246,21 @@ bool axis_in_window(double s, double r, double cell, int f) {
   return d >= -h && d < h;
 }
 
+// Twiddle tables exp(-2 pi i k/N) of a device, shared by its contexts (a map server makes
+// one context per request) and freed with the last of them: at most one table per grid and
+// cut size.  Uploaded with a synchronous copy, so any stream may read them afterwards.
+struct TwiddlePool {
+  int contexts = 0;
+  std::map<int, float2*> tables;
+};
+std::mutex g_twiddle_mu;
+std::map<int, TwiddlePool> g_twiddles;   // by device
+
 eels_status twiddles(eels_ctx* ctx, int n, float2** out) {
-  auto it = ctx->tw.find(n);
-  if (it != ctx->tw.end()) {
+  std::lock_guard<std::mutex> lock(g_twiddle_mu);
+  auto& tables = g_twiddles[ctx->device].tables;
+  auto it = tables.find(n);
+  if (it != tables.end()) {
     *out = it->second;
     return EELS_OK;
   }
@@ -225,8 +269,12 @@ eels_status twiddles(eels_ctx* ctx, int n, float2** out) {
   eels::fill_twiddle_tables(n, h.data());
   float2* d = nullptr;
   EELS_CK(cudaMalloc((void**)&d, len * sizeof(float2)));
-  EELS_CK(cudaMemcpy(d, h.data(), len * sizeof(float2), cudaMemcpyHostToDevice));
-  ctx->tw[n] = d;
+  const cudaError_t e = cudaMemcpy(d, h.data(), len * sizeof(float2), cudaMemcpyHostToDevice);
+  if (e != cudaSuccess) {
+    cudaFree(d);
+    return cuda_fail(ctx, e, "twiddle table");
+  }
+  tables[n] = d;
   *out = d;
   return EELS_OK;
 }
@@ -283,6 +331,10 @@ eels_status eels_create(int device, eels_ctx** out) {
   if (cudaSetDevice(device) != cudaSuccess) return EELS_ERR_CUDA;
   eels_ctx* c = new eels_ctx();
   c->device = device;
+  {
+    std::lock_guard<std::mutex> lock(g_twiddle_mu);
+    g_twiddles[device].contexts++;
+  }
   // keep freed stream-ordered allocations cached between calls
   cudaMemPool_t pool;
   if (cudaDeviceGetDefaultMemPool(&pool, device) == cudaSuccess) {
@@ -296,7 +348,14 @@ eels_status eels_create(int device, eels_ctx** out) {
 void eels_destroy(eels_ctx* ctx) {
   if (!ctx) return;
   cudaSetDevice(ctx->device);
-  for (auto& kv : ctx->tw) cudaFree(kv.second);
+  {
+    std::lock_guard<std::mutex> lock(g_twiddle_mu);
+    TwiddlePool& pool = g_twiddles[ctx->device];
+    if (--pool.contexts == 0) {
+      for (auto& kv : pool.tables) cudaFree(kv.second);
+      pool.tables.clear();
+    }
+  }
   for (auto& r : ctx->recs) { cudaEventDestroy(r.a); cudaEventDestroy(r.b); }
   for (auto e : ctx->spare) cudaEventDestroy(e);
   delete ctx;
@@ -522,11 +581,14 @@ eels_status eels_build_smatrix(eels_ctx* ctx, const eels_specimen* spec, const e
   std::vector<int> px(n_in), py(n_in);
   std::vector<float2> amp(n_in, make_float2(1.f, 0.f));
   for (int j = 0; j < n_in; ++j) { px[j] = op->f * bp[j]; py[j] = op->f * bq[j]; }
-  DevBuf<int> dpx, dpy;
-  DevBuf<float2> damp, W, Phi;
-  if ((e = dpx.upload(px.data(), n_in, st)) != cudaSuccess ||
-      (e = dpy.upload(py.data(), n_in, st)) != cudaSuccess ||
-      (e = damp.upload(amp.data(), n_in, st)) != cudaSuccess ||
+  Pack pack;
+  PackPtr<int> dpx, dpy;
+  PackPtr<float2> damp;
+  pack.add(dpx, px);
+  pack.add(dpy, py);
+  pack.add(damp, amp);
+  DevBuf<float2> W, Phi;
+  if ((e = pack.upload(st)) != cudaSuccess ||
       (e = W.alloc((size_t)n_in * n * nh, st)) != cudaSuccess ||
       (e = Phi.alloc((size_t)n_in * n * nh, st)) != cudaSuccess)
     return bail(cuda_fail(ctx, e, "S_in work buffers"));
@@ -712,44 +774,26 @@ eels_status map_window(eels_ctx* ctx, const eels_smatrix* sm, const eels_transit
   for (int s = 0; s < S; ++s)
     if (L.xcnt[s] > 0 && L.ycnt[s] > 0) slice_sites[tr->slice[s]].push_back(s);
 
-  DevBuf<float2> dH, Sout, W, Phi, M, axT, ayT, damp;
-  DevBuf<int> dwx, dwy, dxoff, dxcnt, dxlist, dyoff, dycnt, dylist, dpx, dpy, dbp, dbq;
+  DevBuf<float2> dH, Sout, W, Phi, M, axT, ayT;
   DevBuf<double> dmap;
+  Pack pack;
+  PackPtr<float2> damp, pH;
+  PackPtr<int> dwx, dwy, dxoff, dxcnt, dxlist, dyoff, dycnt, dylist, dpx, dpy, dbp, dbq, dslot;
   const float2* H = (const float2*)tr->H;
   const int h_mul = tr->h_shared ? 0 : 1;
   const size_t hcount = (size_t)(tr->h_shared ? 1 : S) * T * w * w;
-  if (!tr->on_device) {
-    EELS_CK(dH.upload((const float2*)tr->H, hcount, st));
-    H = dH.p;
-  }
-  EELS_CK(dwx.upload(tr->win_x0, S, st));
-  EELS_CK(dwy.upload(tr->win_y0, S, st));
-#ifdef STEM_CHECK
-  if (ctx->check_test) {   // origin N/2 for the first site some probe reaches; a periodic
-    int s0 = 0;              // walk from there still stays inside the plane
-    while (s0 < S && (L.xcnt[s0] == 0 || L.ycnt[s0] == 0)) ++s0;
-    if (s0 < S) {
-      const int bad = nh;
-      EELS_CK(cudaMemcpyAsync(dwx.p + s0, &bad, sizeof(int), cudaMemcpyHostToDevice, st));
-      EELS_CK(cudaStreamSynchronize(st));
-    }
-  }
-#endif
-  EELS_CK(dxoff.upload(L.xoff.data(), S, st));
-  EELS_CK(dxcnt.upload(L.xcnt.data(), S, st));
-  EELS_CK(dxlist.upload(L.xlist.data(), L.xlist.size(), st));
-  EELS_CK(dyoff.upload(L.yoff.data(), S, st));
-  EELS_CK(dycnt.upload(L.ycnt.data(), S, st));
-  EELS_CK(dylist.upload(L.ylist.data(), L.ylist.size(), st));
-  EELS_CK(dbp.upload(sm->bp.data(), n_in, st));
-  EELS_CK(dbq.upload(sm->bq.data(), n_in, st));
-  // phase tables [pos][n_in]: the contractions read along the beams
-  EELS_CK(axT.alloc((size_t)n_in * win.nx, st));
-  EELS_CK(ayT.alloc((size_t)n_in * win.ny, st));
-  EELS_CK(eels::launch_phase_table(axT.p, dbp.p, n_in, f, sm->cell, sc->x0, sc->step_x, win.nx,
-                                   st, 1, win.ix0));
-  EELS_CK(eels::launch_phase_table(ayT.p, dbq.p, n_in, f, sm->cell, sc->y0, sc->step_y, win.ny,
-                                   st, 1, win.iy0));
+  const bool pack_h = !tr->on_device && hcount * sizeof(float2) <= (1u << 18);
+  if (pack_h) pack.add(pH, H, hcount);
+  pack.add(dwx, tr->win_x0, S);
+  pack.add(dwy, tr->win_y0, S);
+  pack.add(dxoff, L.xoff);
+  pack.add(dxcnt, L.xcnt);
+  pack.add(dxlist, L.xlist);
+  pack.add(dyoff, L.yoff);
+  pack.add(dycnt, L.ycnt);
+  pack.add(dylist, L.ylist);
+  pack.add(dbp, sm->bp);
+  pack.add(dbq, sm->bq);
 
   // reached sites of all slices, slice after slice
   std::vector<int> slot_all, site_off(n_z + 1, 0);
@@ -760,8 +804,7 @@ eels_status map_window(eels_ctx* ctx, const eels_smatrix* sm, const eels_transit
     max_sites = std::max(max_sites, (int)slice_sites[i].size());
   }
   site_off[n_z] = (int)slot_all.size();
-  DevBuf<int> dslot;
-  EELS_CK(dslot.upload(slot_all.data(), slot_all.size(), st));
+  pack.add(dslot, slot_all);
 
   // detector plane waves at the exit surface, carried back by conj(P) first:
   // beta_d(n_z - 1) = conj(P(k_d)) |k_d>
@@ -775,14 +818,16 @@ eels_status map_window(eels_ctx* ctx, const eels_smatrix* sm, const eels_transit
     a -= 2.0 * std::floor(0.5 * a);
     amp[d] = make_float2((float)std::cos(kPi * a), (float)std::sin(kPi * a));
   }
-  EELS_CK(dpx.upload(px.data(), n_out, st));
-  EELS_CK(dpy.upload(py.data(), n_out, st));
-  EELS_CK(damp.upload(amp.data(), n_out, st));
+  pack.add(dpx, px);
+  pack.add(dpy, py);
+  pack.add(damp, amp);
   EELS_CK(Sout.alloc((size_t)n_out * plane, st));
   EELS_CK(W.alloc((size_t)n_out * n * nh, st));
   EELS_CK(Phi.alloc((size_t)n_out * n * nh, st));
-  EELS_CK(dmap.alloc((size_t)n_map, st));
-  EELS_CK(cudaMemsetAsync(dmap.p, 0, sizeof(double) * n_map, st));
+  // the map and, behind it, the call's status word
+  EELS_CK(dmap.alloc((size_t)n_map + 1, st));
+  EELS_CK(cudaMemsetAsync(dmap.p, 0, sizeof(double) * (n_map + 1), st));
+  int* dstatus = reinterpret_cast<int*>(dmap.p + n_map);
   // checkpointed S-matrix: forward work arrays and one segment of K depths of S_in
   const int K = sm->ckpt_k;
   DevBuf<float2> Wf, Phif, seg;
@@ -873,11 +918,11 @@ eels_status map_window(eels_ctx* ctx, const eels_smatrix* sm, const eels_transit
                                                        ctx->operand_budget / per_site));
   if (ctx->batch_sites > 0) sb = std::min(sb, ctx->batch_sites);
   DevBuf<float> A1, B1, M1, B2, AY, BY, BV;
-  DevBuf<int> dzs, dzt, dab1, dbb1, dnv1, dab2, dbb2, dnv2, dstatus, daby, dnvy, dnry;
+  PackPtr<int> dzs, dzt, dab1, dbb1, dnv1, dab2, dbb2, dnv2, daby, dnvy, dnry;
   DevBuf<double> dscratch;
   std::vector<int> zs_all, zt_all, nv2_all, nr_all;
   std::vector<int> pv_all[2], py_all[2];   // [0]: 256-column tiles, [1]: 128-column tiles
-  DevBuf<int> dtile_v[2], dtile_y[2];
+  PackPtr<int> dtile_v[2], dtile_y[2];
   if (tc) {
     for (int s : slot_all) {
       nr_all.push_back(L.xcnt[s] * L.ycnt[s]);
@@ -903,27 +948,25 @@ eels_status map_window(eels_ctx* ctx, const eels_smatrix* sm, const eels_transit
     }
     std::vector<int> ab1(sb * T), bb1(sb * T), nv1(sb * T, k2p), ab2(sb * T), bb2(sb * T);
     for (int z = 0; z < sb * T; ++z) { ab1[z] = z / T; bb1[z] = z; ab2[z] = z; bb2[z] = z / T; }
-    EELS_CK(dzs.upload(zs_all.data(), zs_all.size(), st));
-    EELS_CK(dzt.upload(zt_all.data(), zt_all.size(), st));
-    EELS_CK(dnv2.upload(nv2_all.data(), nv2_all.size(), st));
+    pack.add(dzs, zs_all);
+    pack.add(dzt, zt_all);
+    pack.add(dnv2, nv2_all);
     for (int nw = 0; nw < 2; ++nw) {
-      EELS_CK(dtile_v[nw].upload(pv_all[nw].data(), pv_all[nw].size(), st));
-      EELS_CK(dtile_y[nw].upload(py_all[nw].data(), py_all[nw].size(), st));
+      pack.add(dtile_v[nw], pv_all[nw]);
+      pack.add(dtile_y[nw], py_all[nw]);
     }
-    EELS_CK(dab1.upload(ab1.data(), ab1.size(), st));
-    EELS_CK(dbb1.upload(bb1.data(), bb1.size(), st));
-    EELS_CK(dnv1.upload(nv1.data(), nv1.size(), st));
-    EELS_CK(dab2.upload(ab2.data(), ab2.size(), st));
-    EELS_CK(dbb2.upload(bb2.data(), bb2.size(), st));
-    EELS_CK(dstatus.alloc(1, st));
-    EELS_CK(cudaMemsetAsync(dstatus.p, 0, sizeof(int), st));
+    pack.add(dab1, ab1);
+    pack.add(dbb1, bb1);
+    pack.add(dnv1, nv1);
+    pack.add(dab2, ab2);
+    pack.add(dbb2, bb2);
     EELS_CK(A1.alloc((size_t)vf * sb * n_out * k1p, st));
     if (need_pr) {
       std::vector<int> aby(sb), nvy(sb, k1p);
       for (int q = 0; q < sb; ++q) aby[q] = q;
-      EELS_CK(daby.upload(aby.data(), aby.size(), st));
-      EELS_CK(dnvy.upload(nvy.data(), nvy.size(), st));
-      EELS_CK(dnry.upload(nr_all.data(), nr_all.size(), st));
+      pack.add(daby, aby);
+      pack.add(dnvy, nvy);
+      pack.add(dnry, nr_all);
       EELS_CK(AY.alloc((size_t)vf * sb * nr_cap * k2p, st));
       EELS_CK(BY.alloc((size_t)vf * sb * k1p * k2p, st));
       EELS_CK(BV.alloc((size_t)vf * sb * T * 2 * nr_cap * k1p, st));
@@ -935,6 +978,31 @@ eels_status map_window(eels_ctx* ctx, const eels_smatrix* sm, const eels_transit
     }
     if (tune) EELS_CK(dscratch.alloc((size_t)n_map, st));
   }
+  EELS_CK(pack.upload(st));
+  if (pack_h) {
+    H = pH.p;
+  } else if (!tr->on_device) {
+    EELS_CK(dH.upload((const float2*)tr->H, hcount, st));
+    H = dH.p;
+  }
+#ifdef STEM_CHECK
+  if (ctx->check_test) {   // origin N/2 for the first site some probe reaches; a periodic
+    int s0 = 0;              // walk from there still stays inside the plane
+    while (s0 < S && (L.xcnt[s0] == 0 || L.ycnt[s0] == 0)) ++s0;
+    if (s0 < S) {
+      const int bad = nh;
+      EELS_CK(cudaMemcpyAsync(dwx.p + s0, &bad, sizeof(int), cudaMemcpyHostToDevice, st));
+      EELS_CK(cudaStreamSynchronize(st));
+    }
+  }
+#endif
+  // phase tables [pos][n_in]: the contractions read along the beams
+  EELS_CK(axT.alloc((size_t)n_in * win.nx, st));
+  EELS_CK(ayT.alloc((size_t)n_in * win.ny, st));
+  EELS_CK(eels::launch_phase_table(axT.p, dbp.p, n_in, f, sm->cell, sc->x0, sc->step_x, win.nx,
+                                   st, 1, win.ix0));
+  EELS_CK(eels::launch_phase_table(ayT.p, dbq.p, n_in, f, sm->cell, sc->y0, sc->step_y, win.ny,
+                                   st, 1, win.iy0));
 
   {
     Prof pr(ctx, "init_plane_waves", st);
@@ -983,7 +1051,7 @@ eels_status map_window(eels_ctx* ctx, const eels_smatrix* sm, const eels_transit
       b.yoff = dyoff.p; b.ycnt = dycnt.p; b.ylist = dylist.p; b.nr_cap = nr_cap;
       b.a_batch1 = dab1.p; b.b_batch1 = dbb1.p; b.n_valid1 = dnv1.p;
       b.a_batch2 = dab2.p; b.b_batch2 = dbb2.p; b.n_valid2 = dnv2.p + (int64_t)q0 * T;
-      b.map = map; b.status = dstatus.p;
+      b.map = map; b.status = dstatus;
       b.wait_cycles = ctx->wait_test > 0 ? 1000LL * ctx->wait_test : 0;
       b.withhold = ctx->wait_test > 0 ? 1 : 0;
       b.AY = AY.p; b.BY = BY.p; b.BV = BV.p; b.a_batch_y = daby.p; b.n_valid_y = dnvy.p;
@@ -1234,26 +1302,22 @@ eels_status map_window(eels_ctx* ctx, const eels_smatrix* sm, const eels_transit
   // device status: bit 1 a bounded tensor-core wait timed out, bit 2 the map holds NaN or
   // Inf (the sentinel), bit 4 a check of the bounds-checked build failed; read once the
   // work is done
-  if (!dstatus.p) {
-    EELS_CK(dstatus.alloc(1, st));
-    EELS_CK(cudaMemsetAsync(dstatus.p, 0, sizeof(int), st));
-  }
-  EELS_CK(eels::launch_scale_check(dmap.p, n_map, scale, dstatus.p, st));
-  EELS_CK(collect_checks(dstatus.p, st));
-  {
-    int flag = 0;
-    EELS_CK(cudaMemcpyAsync(&flag, dstatus.p, sizeof(int), cudaMemcpyDeviceToHost, st));
-    EELS_CK(cudaStreamSynchronize(st));
-    if (flag & 4) return fail(ctx, EELS_ERR_BOUNDS, "a bounds check of the debug build failed");
-    if (flag & 1) return fail(ctx, EELS_ERR_TIMEOUT, "tensor-core pipeline wait timed out");
-    nonfinite = (flag & 2) != 0;
-  }
-  if (map_on_device) {
+  EELS_CK(eels::launch_scale_check(dmap.p, n_map, scale, dstatus, st));
+  EELS_CK(collect_checks(dstatus, st));
+  // a host map comes back together with the status word
+  std::vector<double> back(map_on_device ? 1 : (size_t)n_map + 1);
+  EELS_CK(cudaMemcpyAsync(back.data(), map_on_device ? dmap.p + n_map : dmap.p,
+                          sizeof(double) * back.size(), cudaMemcpyDeviceToHost, st));
+  EELS_CK(cudaStreamSynchronize(st));
+  int flag = 0;
+  std::memcpy(&flag, &back.back(), sizeof(int));
+  if (flag & 4) return fail(ctx, EELS_ERR_BOUNDS, "a bounds check of the debug build failed");
+  if (flag & 1) return fail(ctx, EELS_ERR_TIMEOUT, "tensor-core pipeline wait timed out");
+  nonfinite = (flag & 2) != 0;
+  if (map_on_device)
     EELS_CK(cudaMemcpyAsync(map_out, dmap.p, sizeof(double) * n_map, cudaMemcpyDeviceToDevice, st));
-  } else {
-    EELS_CK(cudaMemcpyAsync(map_out, dmap.p, sizeof(double) * n_map, cudaMemcpyDeviceToHost, st));
-    EELS_CK(cudaStreamSynchronize(st));
-  }
+  else
+    std::memcpy(map_out, back.data(), sizeof(double) * n_map);
   if (nonfinite) return fail(ctx, EELS_ERR_NONFINITE, "the map holds NaN or Inf values");
   return EELS_OK;
 }

@@ -83,6 +83,7 @@ struct eels_server {
   int running = 0;                  // admitted requests not yet finished
   bool stop = false;
   double t0 = 0, t_first = -1, t_last = 0;
+  eels_ctx* base = nullptr;         // keeps the device's shared tables between requests
   std::thread admitter;
   std::vector<std::thread> threads;
 };
@@ -247,6 +248,11 @@ eels_status eels_server_create(int device, int64_t hbm_budget, int slots, eels_s
   if (cudaGetDeviceCount(&count) != cudaSuccess || device < 0 || device >= count)
     return EELS_ERR_CUDA;
   eels_server* sv = new eels_server();
+  const eels_status made = eels_create(device, &sv->base);
+  if (made != EELS_OK) {
+    delete sv;
+    return made;
+  }
   sv->device = device;
   sv->budget = hbm_budget;
   sv->slots = slots;
@@ -419,6 +425,7 @@ void eels_server_destroy(eels_server* sv) {
   // admitted requests run to completion; the admitter has stopped adding threads
   for (auto& t : sv->threads) t.join();
   for (auto& kv : sv->requests) delete kv.second;
+  eels_destroy(sv->base);
   delete sv;
 }
 
