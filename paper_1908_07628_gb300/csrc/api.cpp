@@ -592,12 +592,13 @@ eels_status eels_build_smatrix(eels_ctx* ctx, const eels_specimen* spec, const e
       (e = W.alloc((size_t)n_in * n * nh, st)) != cudaSuccess ||
       (e = Phi.alloc((size_t)n_in * n * nh, st)) != cudaSuccess)
     return bail(cuda_fail(ctx, e, "S_in work buffers"));
-  {
+  const int K = sm->ckpt_k;
+  const eels::PlaneWaves plane_waves{dpx.p, dpy.p, damp.p};
+  if (K) {   // the checkpoint of depth 0 holds them; otherwise the first row pass forms them
     Prof pr(ctx, "init_plane_waves", st);
     if ((e = eels::launch_init_plane_waves(W.p, n, n_in, dpx.p, dpy.p, damp.p, tw, st)) != cudaSuccess)
       return bail(cuda_fail(ctx, e, "init plane waves"));
   }
-  const int K = sm->ckpt_k;
   for (int i = 0; i < n_z; ++i) {
     const bool last = (i == n_z - 1) && !sm->s_exit;   // the exit plane needs one more half step
     if (K && i % K == 0) {   // checkpoint psi_j(i), the row pass input of slice i
@@ -610,7 +611,7 @@ eels_status eels_build_smatrix(eels_ctx* ctx, const eels_specimen* spec, const e
       Prof pr(ctx, "row_pass", st);
       e = launch_row_pass(n, n_in, W.p, Phi.p, sm->t + (int64_t)i * n * n, 0, K ? 0 : 1,
                           K ? nullptr : sm->s_in + (int64_t)i * n_in * plane, K ? 0 : n_in, plane,
-                          last ? 0 : 1, tw, st);
+                          last ? 0 : 1, tw, st, i == 0 && !K ? &plane_waves : nullptr);
     }
     if (e != cudaSuccess) return bail(cuda_fail(ctx, e, "row pass"));
     if (!last) {
@@ -1004,7 +1005,8 @@ eels_status map_window(eels_ctx* ctx, const eels_smatrix* sm, const eels_transit
   EELS_CK(eels::launch_phase_table(ayT.p, dbq.p, n_in, f, sm->cell, sc->y0, sc->step_y, win.ny,
                                    st, 1, win.iy0));
 
-  {
+  const eels::PlaneWaves plane_waves{dpx.p, dpy.p, damp.p};
+  if (ctx->sout_scheme == EELS_SOUT_INVERSE) {
     Prof pr(ctx, "init_plane_waves", st);
     EELS_CK(eels::launch_init_plane_waves(W.p, n, n_out, dpx.p, dpy.p, damp.p, tw, st));
   }
@@ -1231,7 +1233,7 @@ eels_status map_window(eels_ctx* ctx, const eels_smatrix* sm, const eels_transit
       if (store || i > 0) {
         Prof pr(ctx, "row_pass_adjoint", st);
         EELS_CK(launch_row_pass(n, n_out, W.p, Phi.p, t_of(i), 1, store, Sout.p, n_out, plane,
-                                i > 0 ? 1 : 0, tw, st));
+                                i > 0 ? 1 : 0, tw, st, i == n_z - 1 ? &plane_waves : nullptr));
       }
       if ((rs = contract_depth(i)) != EELS_OK) return rs;
       if (i > 0) {

@@ -41,12 +41,20 @@ cudaError_t launch_propagator_table(float2* ptab, int n, double cell, double lam
 cudaError_t launch_init_plane_waves(float2* W, int n, int n_waves, const int* px, const int* py,
                                     const float2* amp, const float2* tw, cudaStream_t s);
 
+// Plane waves as k_init_plane_waves writes them (device arrays).
+struct PlaneWaves {
+  const int* px;
+  const int* py;
+  const float2* amp;
+};
 // Row pass of one slice step for n_waves waves (see multislice.cu).
 //   store_mode 0: none; 1: store Dec(t psi) (S_in); 2: store Dec(psi) before the
 //   transmission (S_out).  Only waves < s_waves are stored, at S + wave*s_stride.
+//   start: the input is these plane waves; W is not read.
 cudaError_t launch_row_pass(int n, int n_waves, const float2* W, float2* Phi, const float2* t_slice,
                             int conj_t, int store_mode, float2* S, int s_waves, int64_t s_stride,
-                            int fft_out, const float2* tw, cudaStream_t s);
+                            int fft_out, const float2* tw, cudaStream_t s,
+                            const PlaneWaves* start = nullptr);
 
 // Column pass: FFT_y, crop to the band box, multiply by Ptab (or conj), and then
 //   mode 0: zero-pad and inverse FFT_y back into W;

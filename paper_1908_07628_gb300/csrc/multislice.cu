@@ -56,9 +56,11 @@ struct RowSmem {
 // (ncu, 1024: 69 %, FMA pipe 55 %, shared-memory wavefronts 66 %, DRAM 45 %).  Adjoint pass
 // with the S_out store, us per wave, before -> now: 1024: 3.22 -> 2.95, 768: 1.83 -> 1.55,
 // 512: 0.58 -> 0.57, 384: 1.00 -> 0.48 (four stages and three exchanges before).
-template <int N, bool CONJ>
+// START: the waves are plane waves, formed here instead of being read (the first slice of a
+// sweep; writing them out and reading them back cost a build 4 % of its time).
+template <int N, bool CONJ, bool START>
 __global__ void __launch_bounds__(kRowWarps * 32, row_ctas<N>())
-k_row_pass(const float2* __restrict__ W, float2* __restrict__ Phi,
+k_row_pass(const float2* __restrict__ W, const PlaneWaves start, float2* __restrict__ Phi,
            const float2* __restrict__ t_slice, int store_mode, float2* __restrict__ S,
            int s_waves, int64_t s_stride, int fft_out, const float2* __restrict__ tw,
            int n_waves, int chunk) {
@@ -78,30 +80,48 @@ k_row_pass(const float2* __restrict__ W, float2* __restrict__ Phi,
 
   float2 v[pf::Seqs<N>::E];
   // inputs of the inverse x-FFT: the band box, zero-padded to N
-  auto load = [&](int64_t base) {
+  auto load = [&](int64_t wave) {
+    int col = -1, ky = 0;   // START: the wave's box column (-1: none) and y frequency
+    float2 a = make_float2(0.f, 0.f);
+    if constexpr (START) {
+      const int p = start.px[wave];
+      if (STEM_REQUIRE(p >= -NH && p < NH)) col = p >= 0 ? p : p + NH;
+      ky = start.py[wave];
+      a = start.amp[wave];
+    }
 #pragma unroll
     for (int t = 0; t < PI::PER0; ++t) {
       const int u = lane + 32 * t;
       if ((SEQ * PI::NB0) % 32 == 0 || u < SEQ * PI::NB0) {
-        const float2* src = W + base + (u / PI::NB0) * NH + u % PI::NB0;
+        const int y = y0 + u / PI::NB0, b = u % PI::NB0;
+        const float2* src = W + (wave * N + y) * NH + b;
+        float2 on = make_float2(0.f, 0.f);
+        if constexpr (START) {
+          const int m = ky * y % N;
+          on = cmul(a, cconj(__ldg(tw + (m < 0 ? m + N : m))));   // exp(+2 pi i ky y / N)
+        }
 #pragma unroll
         for (int q = 0; q < PI::R0; ++q) {
           const int at = q * PI::NB0;
-          if (at < NQ) v[t * PI::R0 + q] = src[at];
-          else if (at >= N - NQ) v[t * PI::R0 + q] = src[at - NH];
-          else v[t * PI::R0 + q] = make_float2(0.f, 0.f);
+          float2 x = make_float2(0.f, 0.f);
+          if (at < NQ || at >= N - NQ) {
+            const int i = at < NQ ? at : at - NH;
+            if constexpr (START) x = b + i == col ? on : x;
+            else x = src[i];
+          }
+          v[t * PI::R0 + q] = x;
         }
       }
     }
   };
-  if (w0 < w_end) load(((int64_t)w0 * N + y0) * NH);
+  if (w0 < w_end) load(w0);
   pf::cp_async_wait();
   __syncthreads();
 
   for (int64_t wave = w0; wave < w_end; wave += kRowWarps) {
     const int64_t base = (wave * N + y0) * NH;
-    if (wave != w0) load(base);
-    if (wave + kRowWarps < w_end) {   // the next rows: SEQ * NH values, contiguous
+    if (wave != w0) load(wave);
+    if (!START && wave + kRowWarps < w_end) {   // the next rows: SEQ * NH values, contiguous
       const float2* next = W + base + (int64_t)kRowWarps * N * NH;
 #pragma unroll
       for (int i = lane * 16; i < SEQ * NH; i += 512) prefetch_l2(next + i);
@@ -454,29 +474,29 @@ int wave_chunk(int n_waves, int blocks_x, int width, int resident) {
   return width * (int)std::min<int64_t>(per, 16);
 }
 
-template <int N, bool CONJ>
-cudaError_t row_pass_c(int n_waves, const float2* W, float2* Phi, const float2* t, int store_mode,
-                       float2* S, int s_waves, int64_t s_stride, int fft_out, const float2* tw,
-                       cudaStream_t s) {
+template <int N, bool CONJ, bool START>
+cudaError_t row_pass_c(int n_waves, const float2* W, const PlaneWaves& start, float2* Phi,
+                       const float2* t, int store_mode, float2* S, int s_waves, int64_t s_stride,
+                       int fft_out, const float2* tw, cudaStream_t s) {
   static std::atomic<uint64_t> attr{0};
-  cudaError_t e = smem_attr_once(k_row_pass<N, CONJ>, RowSmem<N>::BYTES, attr);
+  cudaError_t e = smem_attr_once(k_row_pass<N, CONJ, START>, RowSmem<N>::BYTES, attr);
   if (e != cudaSuccess) return e;
   const int gx = N / pf::Seqs<N>::SEQ;
   const int chunk = wave_chunk(n_waves, gx, kRowWarps, sm_count() * row_ctas<N>());
   dim3 grid(gx, (n_waves + chunk - 1) / chunk);
-  k_row_pass<N, CONJ><<<grid, kRowWarps * 32, RowSmem<N>::BYTES, s>>>(
-      W, Phi, t, store_mode, S, s_waves, s_stride, fft_out, tw, n_waves, chunk);
+  k_row_pass<N, CONJ, START><<<grid, kRowWarps * 32, RowSmem<N>::BYTES, s>>>(
+      W, start, Phi, t, store_mode, S, s_waves, s_stride, fft_out, tw, n_waves, chunk);
   return cudaGetLastError();
 }
 
 template <int N>
-cudaError_t row_pass_n(int n_waves, const float2* W, float2* Phi, const float2* t, int conj_t,
-                       int store_mode, float2* S, int s_waves, int64_t s_stride, int fft_out,
-                       const float2* tw, cudaStream_t s) {
-  return conj_t ? row_pass_c<N, true>(n_waves, W, Phi, t, store_mode, S, s_waves, s_stride,
-                                      fft_out, tw, s)
-                : row_pass_c<N, false>(n_waves, W, Phi, t, store_mode, S, s_waves, s_stride,
-                                       fft_out, tw, s);
+cudaError_t row_pass_n(int n_waves, const float2* W, const PlaneWaves* start, float2* Phi,
+                       const float2* t, int conj_t, int store_mode, float2* S, int s_waves,
+                       int64_t s_stride, int fft_out, const float2* tw, cudaStream_t s) {
+  const PlaneWaves pw = start ? *start : PlaneWaves{};
+  const auto fn = conj_t ? (start ? row_pass_c<N, true, true> : row_pass_c<N, true, false>)
+                         : (start ? row_pass_c<N, false, true> : row_pass_c<N, false, false>);
+  return fn(n_waves, W, pw, Phi, t, store_mode, S, s_waves, s_stride, fft_out, tw, s);
 }
 
 template <int N, int MODE>
@@ -599,10 +619,11 @@ void fill_twiddle_tables(int n, float2* h) {
 
 cudaError_t launch_row_pass(int n, int n_waves, const float2* W, float2* Phi, const float2* t,
                             int conj_t, int store_mode, float2* S, int s_waves, int64_t s_stride,
-                            int fft_out, const float2* tw, cudaStream_t s) {
+                            int fft_out, const float2* tw, cudaStream_t s,
+                            const PlaneWaves* start) {
   if (n_waves <= 0) return cudaSuccess;
 #define EELS_CASE(NN) \
-  if (n == NN) return row_pass_n<NN>(n_waves, W, Phi, t, conj_t, store_mode, S, s_waves, s_stride, fft_out, tw, s);
+  if (n == NN) return row_pass_n<NN>(n_waves, W, start, Phi, t, conj_t, store_mode, S, s_waves, s_stride, fft_out, tw, s);
   EELS_FOR_EACH_N(EELS_CASE)
 #undef EELS_CASE
   return cudaErrorInvalidValue;

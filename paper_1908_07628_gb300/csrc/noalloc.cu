@@ -178,7 +178,7 @@ extern "C" eels_status eels_build_smatrix_static(const eels_specimen* spec,
   float2* out = reinterpret_cast<float2*>(s_in);
   for (int j0 = 0; j0 < n_in; j0 += chunk) {
     const int nb = std::min(chunk, n_in - j0);
-    EELS_SCK(eels::launch_init_plane_waves(W, n, nb, dpx + j0, dpy + j0, damp + j0, tw, st));
+    const eels::PlaneWaves plane_waves{dpx + j0, dpy + j0, damp + j0};
     for (int i = 0; i < n_z; ++i) {
       const float* v = spec->vproj + (int64_t)i * n * n;
       if (!spec->vproj_on_device) {
@@ -190,7 +190,7 @@ extern "C" eels_status eels_build_smatrix_static(const eels_specimen* spec,
       const bool last = (i == n_z - 1);
       EELS_SCK(eels::launch_row_pass(n, nb, W, Phi, tsl, 0, 1,
                                      out + ((int64_t)i * n_in + j0) * plane, nb, plane,
-                                     last ? 0 : 1, tw, st));
+                                     last ? 0 : 1, tw, st, i == 0 ? &plane_waves : nullptr));
       if (!last)
         EELS_SCK(eels::launch_col_pass(n, nb, Phi, W, ptab, 0, 0, nullptr, nullptr, nullptr, 0.0,
                                        tw, st));
