@@ -14,6 +14,7 @@
 #include <map>
 #include <mutex>
 #include <string>
+#include <unordered_map>
 #include <vector>
 
 #include <nvtx3/nvToolsExt.h>
@@ -726,6 +727,43 @@ eels_status check_transitions(eels_ctx* ctx, const eels_transitions* tr, const e
 
 namespace {
 
+// Sites with the same probes (equal column and row lists) share a set; set_of[k] is the set
+// of sites[k], set_site[u] a site of set u.  In a crystal most windows hold the whole scan.
+struct ProbeSets {
+  std::vector<int> set_of, set_site;
+};
+
+ProbeSets probe_sets(const SiteLists& L, const std::vector<int>& sites) {
+  auto hash = [](const int* v, int n) {
+    uint64_t h = 1469598103934665603ull ^ (uint64_t)n;
+    for (int i = 0; i < n; ++i) h = (h ^ (uint64_t)(uint32_t)v[i]) * 1099511628211ull;
+    return h;
+  };
+  auto same = [&](int a, int b) {
+    return L.xcnt[a] == L.xcnt[b] && L.ycnt[a] == L.ycnt[b] &&
+           std::equal(&L.xlist[L.xoff[a]], &L.xlist[L.xoff[a]] + L.xcnt[a], &L.xlist[L.xoff[b]]) &&
+           std::equal(&L.ylist[L.yoff[a]], &L.ylist[L.yoff[a]] + L.ycnt[a], &L.ylist[L.yoff[b]]);
+  };
+  ProbeSets P;
+  P.set_of.resize(sites.size());
+  std::unordered_multimap<uint64_t, int> by_hash;
+  for (size_t k = 0; k < sites.size(); ++k) {
+    const int s = sites[k];
+    const uint64_t h = hash(&L.xlist[L.xoff[s]], L.xcnt[s]) * 31 + hash(&L.ylist[L.yoff[s]], L.ycnt[s]);
+    int u = -1;
+    const auto range = by_hash.equal_range(h);
+    for (auto it = range.first; it != range.second && u < 0; ++it)
+      if (same(P.set_site[it->second], s)) u = it->second;
+    if (u < 0) {
+      u = (int)P.set_site.size();
+      P.set_site.push_back(s);
+      by_hash.emplace(h, u);
+    }
+    P.set_of[k] = u;
+  }
+  return P;
+}
+
 // The map over one rectangle of the scan, map_out [n_types][win.ny][win.nx]; the
 // arguments are checked by the callers.
 eels_status map_window(eels_ctx* ctx, const eels_smatrix* sm, const eels_transitions* tr,
@@ -908,18 +946,33 @@ eels_status map_window(eels_ctx* ctx, const eels_smatrix* sm, const eels_transit
   const bool need_pr = tune || chosen == EELS_ASSOC_PROBE_FIRST;
   const int vbytes = tc ? eels::tc_value_bytes(tc_prec) : 4;   // operand bytes per value
   const int vf = vbytes / 4;                                      // ... in floats
-  const int64_t per_site =
+  // probe rows of a set (AY, B2), and a site's other operands
+  const int64_t probe_bytes = vbytes * ((need_pr ? (int64_t)nr_cap * k2p : 0) +
+                                        (need_tr ? (int64_t)2 * nr_cap * k2p : 0));
+  const int64_t site_bytes =
       vbytes * ((int64_t)n_out * k1p +
-           (need_pr ? (int64_t)nr_cap * k2p + (int64_t)k1p * k2p + (int64_t)T * 2 * nr_cap * k1p
-                    : 0) +
-           (need_tr ? (int64_t)T * 2 * n_in * k1p + (int64_t)T * n_out * k2p +
-                          (int64_t)2 * nr_cap * k2p
-                    : 0));
-  int sb = (int)std::max<int64_t>(1, std::min<int64_t>(std::max(max_sites, 1),
-                                                       ctx->operand_budget / per_site));
+           (need_pr ? (int64_t)k1p * k2p + (int64_t)T * 2 * nr_cap * k1p : 0) +
+           (need_tr ? (int64_t)T * 2 * n_in * k1p + (int64_t)T * n_out * k2p : 0));
+  // Probe rows do not depend on the depth: where at least every second site repeats the
+  // probes of another and the sets take at most a quarter of the operand budget, they are
+  // gathered once for the whole map, otherwise per site with each batch (the 80 A sphere:
+  // nearly every site has its own probes).
+  ProbeSets sets;
+  int n_sets = 0;
+  if (tc) {
+    sets = probe_sets(L, slot_all);
+    const int64_t u = (int64_t)sets.set_site.size();
+    if (2 * u <= (int64_t)slot_all.size() && 4 * u * probe_bytes <= ctx->operand_budget &&
+        u * probe_bytes + site_bytes <= ctx->operand_budget && u <= 65535)
+      n_sets = (int)u;
+  }
+  const int64_t per_site = site_bytes + (n_sets ? 0 : probe_bytes);
+  int sb = (int)std::max<int64_t>(1, std::min<int64_t>(
+      std::max(max_sites, 1), (ctx->operand_budget - n_sets * probe_bytes) / per_site));
   if (ctx->batch_sites > 0) sb = std::min(sb, ctx->batch_sites);
   DevBuf<float> A1, B1, M1, B2, AY, BY, BV;
   PackPtr<int> dzs, dzt, dab1, dbb1, dnv1, dab2, dbb2, dnv2, daby, dnvy, dnry;
+  PackPtr<int> dset, dset_z, dset_site;
   DevBuf<double> dscratch;
   std::vector<int> zs_all, zt_all, nv2_all, nr_all;
   std::vector<int> pv_all[2], py_all[2];   // [0]: 256-column tiles, [1]: 128-column tiles
@@ -961,6 +1014,13 @@ eels_status map_window(eels_ctx* ctx, const eels_smatrix* sm, const eels_transit
     pack.add(dnv1, nv1);
     pack.add(dab2, ab2);
     pack.add(dbb2, bb2);
+    if (n_sets) {
+      std::vector<int> set_z;
+      for (int u : sets.set_of) set_z.insert(set_z.end(), T, u);
+      pack.add(dset, sets.set_of);
+      pack.add(dset_z, set_z);
+      pack.add(dset_site, sets.set_site);
+    }
     EELS_CK(A1.alloc((size_t)vf * sb * n_out * k1p, st));
     if (need_pr) {
       std::vector<int> aby(sb), nvy(sb, k1p);
@@ -968,14 +1028,14 @@ eels_status map_window(eels_ctx* ctx, const eels_smatrix* sm, const eels_transit
       pack.add(daby, aby);
       pack.add(dnvy, nvy);
       pack.add(dnry, nr_all);
-      EELS_CK(AY.alloc((size_t)vf * sb * nr_cap * k2p, st));
+      EELS_CK(AY.alloc((size_t)vf * (n_sets ? n_sets : sb) * nr_cap * k2p, st));
       EELS_CK(BY.alloc((size_t)vf * sb * k1p * k2p, st));
       EELS_CK(BV.alloc((size_t)vf * sb * T * 2 * nr_cap * k1p, st));
     }
     if (need_tr) {
       EELS_CK(B1.alloc((size_t)vf * sb * T * 2 * n_in * k1p, st));
       EELS_CK(M1.alloc((size_t)vf * sb * T * n_out * k2p, st));
-      EELS_CK(B2.alloc((size_t)vf * sb * 2 * nr_cap * k2p, st));
+      EELS_CK(B2.alloc((size_t)vf * (n_sets ? n_sets : sb) * 2 * nr_cap * k2p, st));
     }
     if (tune) EELS_CK(dscratch.alloc((size_t)n_map, st));
   }
@@ -1009,6 +1069,16 @@ eels_status map_window(eels_ctx* ctx, const eels_smatrix* sm, const eels_transit
   if (ctx->sout_scheme == EELS_SOUT_INVERSE) {
     Prof pr(ctx, "init_plane_waves", st);
     EELS_CK(eels::launch_init_plane_waves(W.p, n, n_out, dpx.p, dpy.p, damp.p, tw, st));
+  }
+  if (n_sets) {
+    eels::TcBatch b{};
+    b.prec = tc_prec; b.n_in = n_in; b.k2p = k2p; b.nr_cap = nr_cap; b.n_sets = n_sets;
+    b.axT = axT.p; b.ayT = ayT.p; b.n_sx = win.nx; b.n_sy = win.ny;
+    b.xoff = dxoff.p; b.xcnt = dxcnt.p; b.xlist = dxlist.p;
+    b.yoff = dyoff.p; b.ycnt = dycnt.p; b.ylist = dylist.p;
+    b.AY = AY.p; b.B2 = B2.p;
+    Prof pr(ctx, "tc_gather_sets", st);
+    EELS_CK(eels::tc_gather_sets(b, dset_site.p, st));
   }
   eels::WindowLists wl{dxoff.p, dxcnt.p, dxlist.p, dyoff.p, dycnt.p, dylist.p, L.max_nr};
   // tensor-core contraction of slice i with one grouping, accumulated into `map`
@@ -1057,6 +1127,9 @@ eels_status map_window(eels_ctx* ctx, const eels_smatrix* sm, const eels_transit
       b.wait_cycles = ctx->wait_test > 0 ? 1000LL * ctx->wait_test : 0;
       b.withhold = ctx->wait_test > 0 ? 1 : 0;
       b.AY = AY.p; b.BY = BY.p; b.BV = BV.p; b.a_batch_y = daby.p; b.n_valid_y = dnvy.p;
+      b.n_sets = n_sets;
+      b.set_of = n_sets ? dset.p + q0 : nullptr;
+      b.set_of_z = n_sets ? dset_z.p + (int64_t)q0 * T : nullptr;
       b.m_valid_y = dnry.p ? dnry.p + q0 : nullptr;
       const bool bf = tc_prec == EELS_TC_BF16X3;
       if (assoc == EELS_ASSOC_PROBE_FIRST) {

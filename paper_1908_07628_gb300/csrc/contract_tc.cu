@@ -821,6 +821,22 @@ cudaError_t make_map(CUtensorMap* map, void* base, int k, int rows, int batch, i
   return r == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
+// probe rows of `count` sites, for GEMM 2 (B2) and GEMM-Y (AY)
+template <int PREC>
+cudaError_t gather_probe_impl(const TcBatch& b, const int* site, int count, cudaStream_t st) {
+  k_gather_probe<PREC><<<dim3(b.nr_cap, count), 256, 0, st>>>(
+      b.axT, b.ayT, b.n_in, b.n_sx, b.n_sy, site, b.xoff, b.xcnt, b.xlist, b.yoff, b.ycnt, b.ylist,
+      b.nr_cap, b.B2, b.k2p);
+  return cudaGetLastError();
+}
+template <int PREC>
+cudaError_t gather_arows_impl(const TcBatch& b, const int* site, int count, cudaStream_t st) {
+  k_gather_arows<PREC><<<dim3((b.nr_cap + kArowRows - 1) / kArowRows, count), 256, 0, st>>>(
+      b.axT, b.ayT, b.n_in, b.n_sx, b.n_sy, site, b.xoff, b.xcnt, b.xlist, b.yoff, b.ycnt, b.ylist,
+      b.nr_cap, b.AY, b.k2p);
+  return cudaGetLastError();
+}
+
 template <int PREC>
 cudaError_t gather_impl(const TcBatch& b, cudaStream_t st) {
   const int nz = b.n_sites * b.n_types;
@@ -832,10 +848,7 @@ cudaError_t gather_impl(const TcBatch& b, cudaStream_t st) {
                                                           b.z_type, b.H, b.n_types, b.h_mul, b.wx,
                                                           b.wy, b.B1, b.k1p);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  k_gather_probe<PREC><<<dim3(b.nr_cap, b.n_sites), 256, 0, st>>>(
-      b.axT, b.ayT, b.n_in, b.n_sx, b.n_sy, b.slot_site, b.xoff, b.xcnt, b.xlist, b.yoff, b.ycnt, b.ylist,
-      b.nr_cap, b.B2, b.k2p);
-  return cudaGetLastError();
+  return b.n_sets ? cudaSuccess : gather_probe_impl<PREC>(b, b.slot_site, b.n_sites, st);
 }
 
 // Launch of one GEMM over a (gx, gy, gz) tile grid (or its listed tiles): the persistent
@@ -886,7 +899,8 @@ cudaError_t gemm2_impl(const TcBatch& b, cudaStream_t st) {
   if ((e = make_map<PREC>(&mM1, b.M1, b.k2p, b.n_out, b.slots_cap * b.n_types, BM)) !=
       cudaSuccess)
     return e;
-  if ((e = make_map<PREC>(&mB2, b.B2, b.k2p, 2 * b.nr_cap, b.slots_cap, BN)) != cudaSuccess)
+  if ((e = make_map<PREC>(&mB2, b.B2, b.k2p, 2 * b.nr_cap, b.n_sets ? b.n_sets : b.slots_cap,
+                          BN)) != cudaSuccess)
     return e;
   EpiStore es{};
   EpiAbs2 ea{b.z_site, b.z_type, b.xoff, b.xcnt, b.xlist, b.yoff, b.ylist, b.n_sx, b.n_sy,
@@ -894,7 +908,8 @@ cudaError_t gemm2_impl(const TcBatch& b, cudaStream_t st) {
   EpiSpread ey{};
   return launch_gemm<1, PREC, BN>(mM1, mB2, mB2, b.k2p / Prec<PREC>::BK, (2 * b.nr_cap + BN - 1) / BN,
                               (b.n_out + BM - 1) / BM, b.n_sites * b.n_types, b.tiles_v,
-                              b.a_batch2, b.b_batch2, b.n_valid2, nullptr, es, ea, ey, b.status,
+                              b.a_batch2, b.n_sets ? b.set_of_z : b.b_batch2, b.n_valid2, nullptr,
+                              es, ea, ey, b.status,
                               st, b.n_tiles_v, b.wait_cycles, b.withhold);
 }
 
@@ -905,10 +920,8 @@ cudaError_t gather_y_impl(const TcBatch& b, cudaStream_t st) {
   k_gather_sout<PREC><<<dim3((b.n_out + kSoutBeams - 1) / kSoutBeams, b.n_sites), 256, 0, st>>>(
       b.Sout, b.nh, b.n_out, b.w, b.slot_site, b.wx, b.wy, b.A1, b.k1p);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  k_gather_arows<PREC><<<dim3((b.nr_cap + kArowRows - 1) / kArowRows, b.n_sites), 256, 0, st>>>(
-      b.axT, b.ayT, b.n_in, b.n_sx, b.n_sy, b.slot_site, b.xoff, b.xcnt, b.xlist, b.yoff, b.ycnt, b.ylist,
-      b.nr_cap, b.AY, b.k2p);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  if (!b.n_sets && (e = gather_arows_impl<PREC>(b, b.slot_site, b.n_sites, st)) != cudaSuccess)
+    return e;
   dim3 gt((b.k1p / 2 + 31) / 32, (b.k2p / 2 + 31) / 32, b.n_sites);
   k_gather_sin_t<PREC><<<gt, 256, 0, st>>>(b.Sin, b.nh, b.n_in, b.w, b.slot_site, b.wx, b.wy,
                                             b.BY, b.k1p, b.k2p);
@@ -919,7 +932,9 @@ template <int PREC, int BN>
 cudaError_t gemm_y_impl(const TcBatch& b, cudaStream_t st) {
   cudaError_t e;
   CUtensorMap mAY, mBY;
-  if ((e = make_map<PREC>(&mAY, b.AY, b.k2p, b.nr_cap, b.slots_cap, BM)) != cudaSuccess) return e;
+  if ((e = make_map<PREC>(&mAY, b.AY, b.k2p, b.nr_cap, b.n_sets ? b.n_sets : b.slots_cap, BM)) !=
+      cudaSuccess)
+    return e;
   if ((e = make_map<PREC>(&mBY, b.BY, b.k2p, b.k1p, b.slots_cap, BN)) != cudaSuccess) return e;
   const int64_t pstride = (int64_t)2 * b.nr_cap * b.k1p;
   EpiStore es{nullptr, 0, 0, 0, 0, b.k1p};
@@ -934,8 +949,8 @@ cudaError_t gemm_y_impl(const TcBatch& b, cudaStream_t st) {
                           CU_TENSOR_MAP_SWIZZLE_64B)) != cudaSuccess)
     return e;
   return launch_gemm<2, PREC, BN>(mAY, mBY, mBV, b.k2p / Prec<PREC>::BK, (b.k1p + BN - 1) / BN,
-                              (b.nr_cap + BM - 1) / BM, b.n_sites, b.tiles_y, b.a_batch_y,
-                              b.a_batch_y, b.n_valid_y, b.m_valid_y, es, ea, ey, b.status, st,
+                              (b.nr_cap + BM - 1) / BM, b.n_sites, b.tiles_y,
+                              b.n_sets ? b.set_of : b.a_batch_y, b.a_batch_y, b.n_valid_y, b.m_valid_y, es, ea, ey, b.status, st,
                               b.n_tiles_y, b.wait_cycles, b.withhold);
 }
 
@@ -963,6 +978,18 @@ cudaError_t tc_gather_y(const TcBatch& b, cudaStream_t st) {
   if (b.n_sites <= 0) return cudaSuccess;
   return b.prec == EELS_TC_BF16X3 ? gather_y_impl<EELS_TC_BF16X3>(b, st)
                                   : gather_y_impl<EELS_TC_TF32>(b, st);
+}
+
+cudaError_t tc_gather_sets(const TcBatch& b, const int* set_site, cudaStream_t st) {
+  const bool bf = b.prec == EELS_TC_BF16X3;
+  cudaError_t e = cudaSuccess;
+  if (b.AY)
+    e = bf ? gather_arows_impl<EELS_TC_BF16X3>(b, set_site, b.n_sets, st)
+           : gather_arows_impl<EELS_TC_TF32>(b, set_site, b.n_sets, st);
+  if (e == cudaSuccess && b.B2)
+    e = bf ? gather_probe_impl<EELS_TC_BF16X3>(b, set_site, b.n_sets, st)
+           : gather_probe_impl<EELS_TC_TF32>(b, set_site, b.n_sets, st);
+  return e;
 }
 
 cudaError_t tc_gemm_y(const TcBatch& b, cudaStream_t st) {

@@ -163,6 +163,11 @@ struct TcBatch {
   int n_sites, slots_cap;                 // sites in this batch, buffer capacity in sites
   int k1p, k2p;                           // padded K of GEMM 1 (2 w^2) and GEMM 2 (2 n_in)
   void* A1; void* B1; void* M1; void* B2;
+  // probe rows: 0: AY / B2 hold one set per slot, gathered with the batch; n: one per
+  // distinct probe set of the map, gathered once (tc_gather_sets), slot q's being set_of[q]
+  // and transition z's set_of_z[z]
+  int n_sets;
+  const int* set_of; const int* set_of_z;
   int n_sx, n_sy;
   const int* xoff; const int* xcnt; const int* xlist;
   const int* yoff; const int* ycnt; const int* ylist;
@@ -192,6 +197,8 @@ cudaError_t tc_gather(const TcBatch& b, cudaStream_t s);   // A1, B1, B2 operand
 cudaError_t tc_gemm1(const TcBatch& b, cudaStream_t s);    // M1 = GEMM 1
 cudaError_t tc_gemm2(const TcBatch& b, cudaStream_t s);    // map += sum_d |GEMM 2|^2
 cudaError_t tc_gather_y(const TcBatch& b, cudaStream_t s); // A1, AY, BY
+// AY and / or B2 (where not null) of n_sets probe sets, set u's probes those of site set_site[u]
+cudaError_t tc_gather_sets(const TcBatch& b, const int* set_site, cudaStream_t s);
 cudaError_t tc_gemm_y(const TcBatch& b, cudaStream_t s);   // BV = H_t . (a rows x Sin window)
 cudaError_t tc_gemm_v(const TcBatch& b, cudaStream_t s);   // map += sum_d |A1 x BV|^2
 
