@@ -581,48 +581,77 @@ struct WindowWalk {
   }
 };
 
-// Beams of S_out per block of the S_out gather, and probe rows per block of the
-// probe-row gather: enough loads per thread to cover the memory latency.
-constexpr int kSoutBeams = 4;
-constexpr int kArowRows = 16;
-
-// A1[slot][plane][d][2p + c] = Sout[d][pixel p of the window of site slot_site[slot]];
-// a block takes kSoutBeams beams d of one site.
+// Store the complex values (a, b) at elements e .. e + 3 of a row (e a multiple of 4, the
+// row 16-byte aligned), in every plane: 8 bytes per plane in BF16, 16 in TF32.
 template <int PREC>
-__global__ void k_gather_sout(const float2* __restrict__ Sout, int nh, int n_out, int w,
-                              const int* __restrict__ slot_site, const int* __restrict__ wx,
-                              const int* __restrict__ wy, void* __restrict__ A1, int k1p) {
-  constexpr int PL = Prec<PREC>::PLANES;
-  const int d0 = blockIdx.x * kSoutBeams, slot = blockIdx.y;
+__device__ __forceinline__ void put4(void* base, int64_t plane_stride, int64_t e, float2 a, float2 b) {
+  if constexpr (PREC == EELS_TC_TF32) {
+    float* p = static_cast<float*>(base);
+    const float4 h = make_float4(tc::to_tf32(a.x), tc::to_tf32(a.y), tc::to_tf32(b.x), tc::to_tf32(b.y));
+    *reinterpret_cast<float4*>(p + e) = h;
+    *reinterpret_cast<float4*>(p + plane_stride + e) =
+        make_float4(tc::to_tf32(a.x - h.x), tc::to_tf32(a.y - h.y), tc::to_tf32(b.x - h.z),
+                    tc::to_tf32(b.y - h.w));
+  } else {
+    __nv_bfloat16* p = static_cast<__nv_bfloat16*>(base);
+    uint2 w[2];
+#pragma unroll
+    for (int pl = 0; pl < 2; ++pl)
+      w[pl] = make_uint2(bf16_pair(bf16_part(a.x, pl), bf16_part(a.y, pl)),
+                         bf16_pair(bf16_part(b.x, pl), bf16_part(b.y, pl)));
+    *reinterpret_cast<uint2*>(p + e) = w[0];
+    *reinterpret_cast<uint2*>(p + plane_stride + e) = w[1];
+  }
+}
+
+constexpr int kSoutBeams = 8;   // beams of S_out per block of the S_out gather (one per warp)
+constexpr int kArowRows = 16;   // probe rows per block of the probe-row gather
+
+// A1[slot][plane][d][2p + c] = Sout[d][pixel p of the window of site slot_site[slot]].  One
+// beam d per warp, its lanes over pixel pairs (8-byte stores per plane instead of 4 in
+// BF16), four pairs in flight: with a block per four beams and single pixels a 24-pixel
+// window left most of its last batch of loads empty.
+template <int PREC>
+__global__ void __launch_bounds__(kSoutBeams * 32)
+k_gather_sout(const float2* __restrict__ Sout, int nh, int n_out, int w,
+              const int* __restrict__ slot_site, const int* __restrict__ wx,
+              const int* __restrict__ wy, void* __restrict__ A1, int k1p) {
+  constexpr int PL = Prec<PREC>::PLANES, U = 4;
+  const int d = blockIdx.x * kSoutBeams + (threadIdx.x >> 5), slot = blockIdx.y;
   const int s = slot_site[slot];
   if (!STEM_REQUIRE(s >= 0 && window_ok(wx[s], wy[s], w, nh))) return;   // whole block
-  const int64_t plane = (int64_t)nh * nh;
+  if (d >= n_out) return;
   const int64_t pstride = (int64_t)n_out * k1p;
-  const int64_t rbase = (int64_t)slot * PL * pstride + (int64_t)d0 * k1p;
-  const float2* src = Sout + (int64_t)d0 * plane;
-  const int nb = min(kSoutBeams, n_out - d0);
-  const int P = w * w;
-  WindowWalk walk(wx[s], wy[s], w, nh);
-  for (int p0 = threadIdx.x; p0 < P; p0 += kGatherBatch * blockDim.x) {
-    int off[kGatherBatch];
-    walk.offsets(p0, P, off);
-    float2 v[kSoutBeams][kGatherBatch];
+  const int64_t row = (int64_t)slot * PL * pstride + (int64_t)d * k1p;
+  const float2* src = Sout + (int64_t)d * nh * nh;
+  const int x0 = wx[s], y0 = wy[s], P = w * w, pairs = k1p / 4;   // padding pairs are zero
+  const int dx = 64 % w, dy = 64 / w;
+  int p = 2 * (threadIdx.x & 31), xx = p % w, yy = p / w;   // this lane's pair: pixels p, p + 1
+  auto at = [&](int x, int y) {
+    int gy = y0 + y, gx = x0 + x;
+    if (gy >= nh) gy -= nh;
+    if (gx >= nh) gx -= nh;
+    return gy * nh + gx;
+  };
+  for (; p < 2 * pairs; p += 64 * U) {
+    float2 v[U][2];
 #pragma unroll
-    for (int b = 0; b < kSoutBeams; ++b)
+    for (int u = 0; u < U; ++u) {
+      v[u][0] = v[u][1] = make_float2(0.f, 0.f);
+      const int q = p + 64 * u;
+      if (q < P) v[u][0] = src[at(xx, yy)];
+      if (q + 1 < P) v[u][1] = xx + 1 < w ? src[at(xx + 1, yy)] : src[at(0, yy + 1)];
+      xx += dx;
+      yy += dy;
+      if (xx >= w) {
+        xx -= w;
+        ++yy;
+      }
+    }
 #pragma unroll
-      for (int u = 0; u < kGatherBatch; ++u)
-        v[b][u] = (b < nb && off[u] >= 0) ? src[b * plane + off[u]] : make_float2(0.f, 0.f);
-#pragma unroll
-    for (int b = 0; b < kSoutBeams; ++b)
-#pragma unroll
-      for (int u = 0; u < kGatherBatch; ++u)
-        if (b < nb && off[u] >= 0)
-          put2<PREC>(A1, pstride, rbase + (int64_t)b * k1p + 2 * (p0 + u * (int)blockDim.x),
-                     v[b][u].x, v[b][u].y);
+    for (int u = 0; u < U; ++u)
+      if (p + 64 * u < 2 * pairs) put4<PREC>(A1, pstride, row + 2 * (p + 64 * u), v[u][0], v[u][1]);
   }
-  for (int b = 0; b < nb; ++b)
-    for (int p = P + threadIdx.x; p < k1p / 2; p += blockDim.x)   // K padding
-      put2<PREC>(A1, pstride, rbase + (int64_t)b * k1p + 2 * p, 0.f, 0.f);
 }
 
 // B1[z][plane][2j][2p + c] = H_z[p] Sin[j][p],  B1[z][plane][2j+1] = -i H_z[p] Sin[j][p]
@@ -729,20 +758,22 @@ __global__ void k_gather_arows(const float2* __restrict__ axT, const float2* __r
   const int64_t pstride = (int64_t)nr_cap * k2p;
   const int64_t base = (int64_t)slot * PL * pstride + (int64_t)rb * k2p;
   for (int i0 = 0; i0 < rows; i0 += 4) {
-    for (int j = threadIdx.x; j < k2p / 2; j += blockDim.x) {
-      float2 a[4];
+    for (int j = 2 * threadIdx.x; j < k2p / 2; j += 2 * blockDim.x) {   // beams j and j + 1
+      float2 a[4][2];
 #pragma unroll
       for (int u = 0; u < 4; ++u) {
         const int i = i0 + u;
         const int ix = i < rows ? s_ix[i] : -1, iy = i < rows ? s_iy[i] : -1;
-        a[u] = (ix >= 0 && j < n_in)
-                   ? cmul(axT[(int64_t)ix * n_in + j], ayT[(int64_t)iy * n_in + j])
-                   : make_float2(0.f, 0.f);
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+          a[u][h] = (ix >= 0 && j + h < n_in)
+                        ? cmul(axT[(int64_t)ix * n_in + j + h], ayT[(int64_t)iy * n_in + j + h])
+                        : make_float2(0.f, 0.f);
       }
 #pragma unroll
       for (int u = 0; u < 4; ++u)
         if (i0 + u < rows)
-          put2<PREC>(AY, pstride, base + (int64_t)(i0 + u) * k2p + 2 * j, a[u].x, a[u].y);
+          put4<PREC>(AY, pstride, base + (int64_t)(i0 + u) * k2p + 2 * j, a[u][0], a[u][1]);
     }
   }
 }
