@@ -540,44 +540,37 @@ k_tc_gemm_ws(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUt
   if (!ok && status) atomicExch(status, 1);
 }
 
-// Window gathers: consecutive threads take consecutive window pixels (coalesced).  A
-// thread's pixels p0, p0 + blockDim.x, ... are visited by an incremental walk (the window
-// row and column advance by fixed steps, no division), and each batch of kGatherBatch
-// loads is issued before any of its stores so that the loads overlap.
-constexpr int kGatherBatch = 4;
+// Window gathers: a warp takes one beam's window, its lanes pixel pairs p, p + 1 (p = 2 lane,
+// then steps of 64).  The pair's window row and column advance by fixed steps (no division),
+// and each batch of kPairBatch pairs is loaded before any of its stores.
+constexpr int kPairBatch = 4;
 
-struct WindowWalk {
+struct PairWalk {
   int x0, y0, w, nh, dx, dy, xx, yy;
-  __device__ WindowWalk(int x0_, int y0_, int w_, int nh_)
-      : x0(x0_), y0(y0_), w(w_), nh(nh_), dx(blockDim.x % w_), dy(blockDim.x / w_),
-        xx(threadIdx.x % w_), yy(threadIdx.x / w_) {}
-  // off[u] = plane offset of pixel p0 + u blockDim.x of the periodic window, -1 past P
-  __device__ __forceinline__ void offsets(int p0, int P, int* off) {
+  __device__ PairWalk(int x0_, int y0_, int w_, int nh_, int p)
+      : x0(x0_), y0(y0_), w(w_), nh(nh_), dx(64 % w_), dy(64 / w_), xx(p % w_), yy(p / w_) {}
+  __device__ __forceinline__ int at(int x, int y) const {   // periodic plane offset
+    int gy = y0 + y, gx = x0 + x;
+    if (gy >= nh) gy -= nh;
+    if (gx >= nh) gx -= nh;
+    return gy * nh + gx;
+  }
+  // v[u] = the window's pixels p + 64 u and p + 64 u + 1 of plane, zero from P on
+  __device__ __forceinline__ void load(const float2* __restrict__ plane, int p, int P,
+                                       float2 (*v)[2]) {
 #pragma unroll
-    for (int u = 0; u < kGatherBatch; ++u) {
-      off[u] = -1;
-      if (p0 + u * (int)blockDim.x < P) {
-        int gy = y0 + yy, gx = x0 + xx;
-        if (gy >= nh) gy -= nh;
-        if (gx >= nh) gx -= nh;
-        off[u] = gy * nh + gx;
-        xx += dx;
-        yy += dy;
-        if (xx >= w) {
-          xx -= w;
-          ++yy;
-        }
+    for (int u = 0; u < kPairBatch; ++u) {
+      const int q = p + 64 * u;
+      v[u][0] = v[u][1] = make_float2(0.f, 0.f);
+      if (q < P) v[u][0] = plane[at(xx, yy)];
+      if (q + 1 < P) v[u][1] = xx + 1 < w ? plane[at(xx + 1, yy)] : plane[at(0, yy + 1)];
+      xx += dx;
+      yy += dy;
+      if (xx >= w) {
+        xx -= w;
+        ++yy;
       }
     }
-  }
-  // v[u] = plane[pixel p0 + u blockDim.x of the window], zero past P
-  __device__ __forceinline__ void load(const float2* __restrict__ plane, int p0, int P,
-                                       float2* v) {
-    int off[kGatherBatch];
-    offsets(p0, P, off);
-#pragma unroll
-    for (int u = 0; u < kGatherBatch; ++u)
-      v[u] = off[u] >= 0 ? plane[off[u]] : make_float2(0.f, 0.f);
   }
 };
 
@@ -604,98 +597,80 @@ __device__ __forceinline__ void put4(void* base, int64_t plane_stride, int64_t e
   }
 }
 
-constexpr int kSoutBeams = 8;   // beams of S_out per block of the S_out gather (one per warp)
-constexpr int kArowRows = 16;   // probe rows per block of the probe-row gather
+constexpr int kGatherBeams = 8;   // beams per block of the window gathers (one per warp)
+constexpr int kArowRows = 16;     // probe rows per block of the probe-row gathers
 
-// A1[slot][plane][d][2p + c] = Sout[d][pixel p of the window of site slot_site[slot]].  One
-// beam d per warp, its lanes over pixel pairs (8-byte stores per plane instead of 4 in
-// BF16), four pairs in flight: with a block per four beams and single pixels a 24-pixel
-// window left most of its last batch of loads empty.
+// A1[slot][plane][d][2p + c] = Sout[d][pixel p of the window of site slot_site[slot]].
+// (A block per four beams with single pixels stored 4 bytes at a time in BF16 and left most
+// of a 24-pixel window's last batch of loads empty: 57 % of the copy bandwidth.)
 template <int PREC>
-__global__ void __launch_bounds__(kSoutBeams * 32)
+__global__ void __launch_bounds__(kGatherBeams * 32)
 k_gather_sout(const float2* __restrict__ Sout, int nh, int n_out, int w,
               const int* __restrict__ slot_site, const int* __restrict__ wx,
               const int* __restrict__ wy, void* __restrict__ A1, int k1p) {
-  constexpr int PL = Prec<PREC>::PLANES, U = 4;
-  const int d = blockIdx.x * kSoutBeams + (threadIdx.x >> 5), slot = blockIdx.y;
+  constexpr int PL = Prec<PREC>::PLANES;
+  const int d = blockIdx.x * kGatherBeams + (threadIdx.x >> 5), slot = blockIdx.y;
   const int s = slot_site[slot];
   if (!STEM_REQUIRE(s >= 0 && window_ok(wx[s], wy[s], w, nh))) return;   // whole block
   if (d >= n_out) return;
   const int64_t pstride = (int64_t)n_out * k1p;
   const int64_t row = (int64_t)slot * PL * pstride + (int64_t)d * k1p;
   const float2* src = Sout + (int64_t)d * nh * nh;
-  const int x0 = wx[s], y0 = wy[s], P = w * w, pairs = k1p / 4;   // padding pairs are zero
-  const int dx = 64 % w, dy = 64 / w;
-  int p = 2 * (threadIdx.x & 31), xx = p % w, yy = p / w;   // this lane's pair: pixels p, p + 1
-  auto at = [&](int x, int y) {
-    int gy = y0 + y, gx = x0 + x;
-    if (gy >= nh) gy -= nh;
-    if (gx >= nh) gx -= nh;
-    return gy * nh + gx;
-  };
-  for (; p < 2 * pairs; p += 64 * U) {
-    float2 v[U][2];
+  const int P = w * w;
+  int p = 2 * (threadIdx.x & 31);
+  PairWalk walk(wx[s], wy[s], w, nh, p);
+  for (; p < k1p / 2; p += 64 * kPairBatch) {   // up to the K padding, which is zero
+    float2 v[kPairBatch][2];
+    walk.load(src, p, P, v);
 #pragma unroll
-    for (int u = 0; u < U; ++u) {
-      v[u][0] = v[u][1] = make_float2(0.f, 0.f);
-      const int q = p + 64 * u;
-      if (q < P) v[u][0] = src[at(xx, yy)];
-      if (q + 1 < P) v[u][1] = xx + 1 < w ? src[at(xx + 1, yy)] : src[at(0, yy + 1)];
-      xx += dx;
-      yy += dy;
-      if (xx >= w) {
-        xx -= w;
-        ++yy;
-      }
-    }
-#pragma unroll
-    for (int u = 0; u < U; ++u)
-      if (p + 64 * u < 2 * pairs) put4<PREC>(A1, pstride, row + 2 * (p + 64 * u), v[u][0], v[u][1]);
+    for (int u = 0; u < kPairBatch; ++u)
+      if (p + 64 * u < k1p / 2) put4<PREC>(A1, pstride, row + 2 * (p + 64 * u), v[u][0], v[u][1]);
   }
 }
 
 // B1[z][plane][2j][2p + c] = H_z[p] Sin[j][p],  B1[z][plane][2j+1] = -i H_z[p] Sin[j][p]
 template <int PREC>
-__global__ void k_gather_sin_h(const float2* __restrict__ Sin, int nh, int n_in, int w,
-                               const int* __restrict__ z_site, const int* __restrict__ z_type,
-                               const float2* __restrict__ H, int n_types, int h_mul,
-                               const int* __restrict__ wx, const int* __restrict__ wy,
-                               void* __restrict__ B1, int k1p) {
+__global__ void __launch_bounds__(kGatherBeams * 32)
+k_gather_sin_h(const float2* __restrict__ Sin, int nh, int n_in, int w,
+               const int* __restrict__ z_site, const int* __restrict__ z_type,
+               const float2* __restrict__ H, int n_types, int h_mul,
+               const int* __restrict__ wx, const int* __restrict__ wy,
+               void* __restrict__ B1, int k1p) {
   constexpr int PL = Prec<PREC>::PLANES;
-  const int j = blockIdx.x, z = blockIdx.y;
+  const int j = blockIdx.x * kGatherBeams + (threadIdx.x >> 5), z = blockIdx.y;
   const int s = z_site[z];
   if (!STEM_REQUIRE(s >= 0 && z_type[z] >= 0 && z_type[z] < n_types &&
                     window_ok(wx[s], wy[s], w, nh)))
     return;   // the whole block
-  const int64_t plane = (int64_t)nh * nh;
+  if (j >= n_in) return;
   const int64_t pstride = (int64_t)2 * n_in * k1p;
   const int64_t r0 = (int64_t)z * PL * pstride + (int64_t)(2 * j) * k1p;
   const int64_t r1 = r0 + k1p;
-  const float2* Hz = H + ((int64_t)s * h_mul * n_types + z_type[z]) * w * w;
-  const float2* src = Sin + (int64_t)j * plane;
   const int P = w * w;
-  WindowWalk walk(wx[s], wy[s], w, nh);
-  for (int p0 = threadIdx.x; p0 < P; p0 += kGatherBatch * blockDim.x) {
-    float2 v[kGatherBatch];
-    walk.load(src, p0, P, v);
+  const float2* Hz = H + ((int64_t)s * h_mul * n_types + z_type[z]) * P;
+  const float2* src = Sin + (int64_t)j * nh * nh;
+  int p = 2 * (threadIdx.x & 31);
+  PairWalk walk(wx[s], wy[s], w, nh, p);
+  for (; p < k1p / 2; p += 64 * kPairBatch) {
+    float2 v[kPairBatch][2];
+    walk.load(src, p, P, v);
 #pragma unroll
-    for (int u = 0; u < kGatherBatch; ++u) {
-      const int p = p0 + u * blockDim.x;
-      if (p < P) {
-        const float2 h = cmul(Hz[p], v[u]);
-        put2<PREC>(B1, pstride, r0 + 2 * p, h.x, h.y);
-        put2<PREC>(B1, pstride, r1 + 2 * p, h.y, -h.x);
-      }
+    for (int u = 0; u < kPairBatch; ++u) {
+      const int q = p + 64 * u;
+      if (q >= k1p / 2) continue;
+      float2 y[2];
+#pragma unroll
+      for (int h = 0; h < 2; ++h)   // zero in the K padding
+        y[h] = q + h < P ? cmul(__ldg(Hz + q + h), v[u][h]) : make_float2(0.f, 0.f);
+      put4<PREC>(B1, pstride, r0 + 2 * q, y[0], y[1]);
+      put4<PREC>(B1, pstride, r1 + 2 * q, make_float2(y[0].y, -y[0].x), make_float2(y[1].y, -y[1].x));
     }
-  }
-  for (int p = P + threadIdx.x; p < k1p / 2; p += blockDim.x) {   // K padding
-    put2<PREC>(B1, pstride, r0 + 2 * p, 0.f, 0.f);
-    put2<PREC>(B1, pstride, r1 + 2 * p, 0.f, 0.f);
   }
 }
 
 // B2[slot][plane][2r] = conj(a_r), B2[slot][plane][2r+1] = i conj(a_r),
-// a_r[j] = ax[j][ix(r)] ay[j][iy(r)]
+// a_r[j] = ax[j][ix(r)] ay[j][iy(r)]; a block takes kArowRows probes, its threads (probe,
+// pair of beams).
 template <int PREC>
 __global__ void k_gather_probe(const float2* __restrict__ axT, const float2* __restrict__ ayT,
                                int n_in, int n_sx, int n_sy, const int* __restrict__ slot_site,
@@ -704,27 +679,41 @@ __global__ void k_gather_probe(const float2* __restrict__ axT, const float2* __r
                                const int* __restrict__ ycnt, const int* __restrict__ ylist,
                                int nr_cap, void* __restrict__ B2, int k2p) {
   constexpr int PL = Prec<PREC>::PLANES;
-  const int r = blockIdx.x, slot = blockIdx.y;
+  __shared__ int s_ix[kArowRows], s_iy[kArowRows];
+  const int rb = blockIdx.x * kArowRows, slot = blockIdx.y;
   const int s = slot_site[slot];
   const int nx = xcnt[s], nr = nx * ycnt[s];
-  // rows of N tiles GEMM 2 skips (the widest tile: a narrower one reads no more rows)
-  if (2 * r >= (2 * nr + BN_WIDE - 1) / BN_WIDE * BN_WIDE) return;
-  const int64_t pstride = (int64_t)2 * nr_cap * k2p;
-  const int64_t r0 = (int64_t)slot * PL * pstride + (int64_t)(2 * r) * k2p;
-  const int64_t r1 = r0 + k2p;
-  int ix = 0, iy = 0;
-  if (r < nr) {
-    ix = xlist[xoff[s] + r % nx];
-    iy = ylist[yoff[s] + r / nx];
-    if (!STEM_REQUIRE(ix >= 0 && ix < n_sx && iy >= 0 && iy < n_sy)) ix = iy = 0;
+  // rows up to the end of the N tiles GEMM 2 reads (the widest tile: a narrower one reads
+  // no more rows)
+  const int r_end = min((2 * nr + BN_WIDE - 1) / BN_WIDE * BN_WIDE / 2, nr_cap);
+  if (rb >= r_end) return;   // the same for the whole block
+  if (threadIdx.x < kArowRows) {
+    const int r = rb + threadIdx.x;
+    int ix = -1, iy = -1;    // -1: a zero row
+    if (r < nr) {
+      ix = xlist[xoff[s] + r % nx];
+      iy = ylist[yoff[s] + r / nx];
+      if (!STEM_REQUIRE(ix >= 0 && ix < n_sx && iy >= 0 && iy < n_sy)) ix = iy = -1;
+    }
+    s_ix[threadIdx.x] = ix;
+    s_iy[threadIdx.x] = iy;
   }
-  const float2* axr = axT + (int64_t)ix * n_in;
-  const float2* ayr = ayT + (int64_t)iy * n_in;
-  for (int j = threadIdx.x; j < k2p / 2; j += blockDim.x) {
-    float2 a = make_float2(0.f, 0.f);
-    if (r < nr && j < n_in) a = cmul(axr[j], ayr[j]);
-    put2<PREC>(B2, pstride, r0 + 2 * j, a.x, -a.y);
-    put2<PREC>(B2, pstride, r1 + 2 * j, a.y, a.x);
+  __syncthreads();
+  const int64_t pstride = (int64_t)2 * nr_cap * k2p;
+  const int64_t base = (int64_t)slot * PL * pstride + (int64_t)(2 * rb) * k2p;
+  const int pairs = k2p / 4, total = min(kArowRows, r_end - rb) * pairs;
+  for (int e = threadIdx.x; e < total; e += blockDim.x) {
+    const int i = e / pairs, j = 2 * (e - i * pairs);
+    const int ix = s_ix[i], iy = s_iy[i];
+    float2 a[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h)
+      a[h] = (ix >= 0 && j + h < n_in)
+                 ? cmul(axT[(int64_t)ix * n_in + j + h], ayT[(int64_t)iy * n_in + j + h])
+                 : make_float2(0.f, 0.f);
+    const int64_t r0 = base + (int64_t)(2 * i) * k2p + 2 * j;
+    put4<PREC>(B2, pstride, r0, make_float2(a[0].x, -a[0].y), make_float2(a[1].x, -a[1].y));
+    put4<PREC>(B2, pstride, r0 + k2p, make_float2(a[0].y, a[0].x), make_float2(a[1].y, a[1].x));
   }
 }
 
@@ -855,7 +844,7 @@ cudaError_t make_map(CUtensorMap* map, void* base, int k, int rows, int batch, i
 // probe rows of `count` sites, for GEMM 2 (B2) and GEMM-Y (AY)
 template <int PREC>
 cudaError_t gather_probe_impl(const TcBatch& b, const int* site, int count, cudaStream_t st) {
-  k_gather_probe<PREC><<<dim3(b.nr_cap, count), 256, 0, st>>>(
+  k_gather_probe<PREC><<<dim3((b.nr_cap + kArowRows - 1) / kArowRows, count), 256, 0, st>>>(
       b.axT, b.ayT, b.n_in, b.n_sx, b.n_sy, site, b.xoff, b.xcnt, b.xlist, b.yoff, b.ycnt, b.ylist,
       b.nr_cap, b.B2, b.k2p);
   return cudaGetLastError();
@@ -872,10 +861,10 @@ template <int PREC>
 cudaError_t gather_impl(const TcBatch& b, cudaStream_t st) {
   const int nz = b.n_sites * b.n_types;
   cudaError_t e;
-  k_gather_sout<PREC><<<dim3((b.n_out + kSoutBeams - 1) / kSoutBeams, b.n_sites), 256, 0, st>>>(
+  k_gather_sout<PREC><<<dim3((b.n_out + kGatherBeams - 1) / kGatherBeams, b.n_sites), 256, 0, st>>>(
       b.Sout, b.nh, b.n_out, b.w, b.slot_site, b.wx, b.wy, b.A1, b.k1p);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  k_gather_sin_h<PREC><<<dim3(b.n_in, nz), 256, 0, st>>>(b.Sin, b.nh, b.n_in, b.w, b.z_site,
+  k_gather_sin_h<PREC><<<dim3((b.n_in + kGatherBeams - 1) / kGatherBeams, nz), 256, 0, st>>>(b.Sin, b.nh, b.n_in, b.w, b.z_site,
                                                           b.z_type, b.H, b.n_types, b.h_mul, b.wx,
                                                           b.wy, b.B1, b.k1p);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
@@ -948,7 +937,7 @@ cudaError_t gemm2_impl(const TcBatch& b, cudaStream_t st) {
 template <int PREC>
 cudaError_t gather_y_impl(const TcBatch& b, cudaStream_t st) {
   cudaError_t e;
-  k_gather_sout<PREC><<<dim3((b.n_out + kSoutBeams - 1) / kSoutBeams, b.n_sites), 256, 0, st>>>(
+  k_gather_sout<PREC><<<dim3((b.n_out + kGatherBeams - 1) / kGatherBeams, b.n_sites), 256, 0, st>>>(
       b.Sout, b.nh, b.n_out, b.w, b.slot_site, b.wx, b.wy, b.A1, b.k1p);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   if (!b.n_sets && (e = gather_arows_impl<PREC>(b, b.slot_site, b.n_sites, st)) != cudaSuccess)
