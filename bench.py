@@ -231,8 +231,9 @@ def cpu_oracle_full(wl_name):
 def _algorithmic(wl, n_in, n_out, prof, steps):
     """Algorithmic bytes of the multislice kernels per step of the default (stream)
     scheme.  Row pass: read W and write Phi (N x N/2 each) and store the even samples
-    ((N/2)^2) per wave, plus the slice's t (N^2) once per launch; the last slice of each
-    sweep stores without writing Phi.  Column pass: read Phi, write W.  Complex64."""
+    ((N/2)^2) per wave, plus the slice's t (N^2) once per launch; the first slice of each
+    sweep forms its plane waves instead of reading W, the last stores without writing Phi.
+    Column pass: read Phi, write W.  Complex64."""
     n, nz = wl.n, wl.n_z
     nh = n // 2
     c = 8
@@ -246,8 +247,9 @@ def _algorithmic(wl, n_in, n_out, prof, steps):
     adj = sum((2 * n * nh + (nh * nh if i in work else 0)) * c for i in range(1, nz)) + \
         (last if 0 in work else 0)
     out = {}
-    for name, waves, per_wave in (("row_pass", n_in, (nz - 1) * row + last),
-                                  ("row_pass_adjoint", n_out, adj)):
+    read = n * nh * c
+    for name, waves, per_wave in (("row_pass", n_in, (nz - 1) * row + last - read),
+                                  ("row_pass_adjoint", n_out, adj - read)):
         launches = prof.get(name, {}).get("launches", 0) / steps
         out[name] = ("hbm", waves * per_wave + launches * t)
     for name, waves in (("col_pass", n_in), ("col_pass_adjoint", n_out)):
@@ -709,11 +711,13 @@ def _multislice_bounds(wl, n_in, n_out, prof, steps, peaks, tpk):
     return out
 
 
-# kernels behind one profiling record: a gather record brackets three gather kernels;
-# every step also runs six small kernels outside the records (propagator table, four
-# phase tables, the final scale-and-check of the map)
-KERNELS_PER_RECORD = {"tc_gather_y": 3, "tc_gather": 3}
-UNRECORDED_PER_STEP = 6
+# kernels behind one profiling record: a gather record brackets three gather kernels, two
+# where the probe rows were gathered once for the map (tc_gather_sets); every step also
+# runs four small kernels outside the records (propagator table, two phase tables, the
+# final scale-and-check of the map)
+KERNELS_PER_RECORD = {"tc_gather_y": 3, "tc_gather": 3, "tc_gather_y_shared": 2,
+                      "tc_gather_shared": 2}
+UNRECORDED_PER_STEP = 4
 
 
 def kernel_launches(prof):

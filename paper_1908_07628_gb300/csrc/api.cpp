@@ -255,7 +255,8 @@ struct TwiddlePool {
   std::map<int, float2*> tables;
 };
 std::mutex g_twiddle_mu;
-std::map<int, TwiddlePool> g_twiddles;   // by device
+// by device; never destroyed, so that a context may be destroyed at any time during exit
+std::map<int, TwiddlePool>& g_twiddles = *new std::map<int, TwiddlePool>();
 
 eels_status twiddles(eels_ctx* ctx, int n, float2** out) {
   std::lock_guard<std::mutex> lock(g_twiddle_mu);
@@ -1134,7 +1135,7 @@ eels_status map_window(eels_ctx* ctx, const eels_smatrix* sm, const eels_transit
       const bool bf = tc_prec == EELS_TC_BF16X3;
       if (assoc == EELS_ASSOC_PROBE_FIRST) {
         {
-          Prof pr(ctx, "tc_gather_y", st);
+          Prof pr(ctx, n_sets ? "tc_gather_y_shared" : "tc_gather_y", st);
           EELS_CK(eels::tc_gather_y(b, st));
         }
         {
@@ -1147,7 +1148,7 @@ eels_status map_window(eels_ctx* ctx, const eels_smatrix* sm, const eels_transit
         }
       } else {
         {
-          Prof pr(ctx, "tc_gather", st);
+          Prof pr(ctx, n_sets ? "tc_gather_shared" : "tc_gather", st);
           EELS_CK(eels::tc_gather(b, st));
         }
         {
