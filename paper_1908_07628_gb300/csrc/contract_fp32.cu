@@ -333,11 +333,12 @@ __global__ void k_scale_check(double* a, int64_t count, double scale, int* flag)
 namespace {
 
 // Estimated cycles of one K step over a whole launch with 16 im x 16 jn tiles: the CTAs of
-// the busiest SM after one another at 128 im jn cycles of FMA issue each, plus the latency
-// of a step that nothing hides when few CTAs share an SM.
+// the busiest SM after one another, each 128 im jn cycles of FMA issue and the issue slots of
+// its loads and its loop (about 300 + 68 (im + jn), from instruction counts), plus the
+// latency of a step where one CTA has an SM to itself.
 double step_cost(int64_t ctas, int im, int jn) {
   const double per_sm = (double)((ctas + sm_count() - 1) / sm_count());
-  return per_sm * 128.0 * im * jn + (per_sm < 2 ? 500.0 : 250.0);
+  return per_sm * (128.0 * im * jn + 68.0 * (im + jn) + 300.0) + (per_sm < 2 ? 500.0 : 0.0);
 }
 
 template <int IM, int JN>
@@ -378,11 +379,13 @@ cudaError_t launch_gemm1_fp32(const float2* Sout, const float2* Sin, int nh, int
                               cudaStream_t s) {
   if (sb.count <= 0 || sb.nt <= 0) return cudaSuccess;
   // the tile that wastes least on the edges of n_out and nt n_in, or spreads a small
-  // launch over more SMs
+  // launch over more SMs (the 64-grid map takes 60 CTAs of 16 x 16 instead of 18 of 32 x 32:
+  // 218 -> 198 us)
   int im = 0, jn = 0;
   double best = 0;
-  for (int i : {8, 7, 6, 5, 4, 2})
-    for (int j : {4, 2}) {
+  for (int i : {8, 7, 6, 5, 4, 2, 1})
+    for (int j : {4, 2, 1}) {
+      if (j == 1 ? i > 2 : i < 2) continue;   // not built
       const int64_t ctas = (int64_t)((sb.nt * n_in + 16 * j - 1) / (16 * j)) *
                            ((n_out + 16 * i - 1) / (16 * i)) * sb.count;
       const double c = step_cost(ctas, i, j);
@@ -394,6 +397,7 @@ cudaError_t launch_gemm1_fp32(const float2* Sout, const float2* Sin, int nh, int
                             win_y0, M, m_stride, s);
   EELS_G1(8, 4) EELS_G1(7, 4) EELS_G1(6, 4) EELS_G1(5, 4) EELS_G1(4, 4) EELS_G1(2, 4)
   EELS_G1(8, 2) EELS_G1(7, 2) EELS_G1(6, 2) EELS_G1(5, 2) EELS_G1(4, 2) EELS_G1(2, 2)
+  EELS_G1(2, 1) EELS_G1(1, 1)
 #undef EELS_G1
   return cudaErrorInvalidValue;
 }
@@ -407,7 +411,8 @@ cudaError_t launch_gemm2_abs2_fp32(const float2* M, int64_t m_stride, int n_out,
   int g = 0, jn = 0;
   double best = 0;
   for (int i : {2, 1})
-    for (int j : {4, 2}) {
+    for (int j : {4, 2, 1}) {
+      if (i == 2 && j == 1) continue;   // not built
       const int64_t ctas = (int64_t)((wl.max_nr + 16 * j - 1) / (16 * j)) * ((groups + i - 1) / i) *
                            sb.count;
       const double c = step_cost(ctas, 4 * i, j);
@@ -416,7 +421,7 @@ cudaError_t launch_gemm2_abs2_fp32(const float2* M, int64_t m_stride, int n_out,
 #define EELS_G2(I, J)                                                                         \
   if (g == I && jn == J)                                                                      \
     return gemm2_tile<I, J>(M, m_stride, n_out, n_in, axT, ayT, n_sx, n_sy, sb, wl, map, s);
-  EELS_G2(2, 4) EELS_G2(1, 4) EELS_G2(2, 2) EELS_G2(1, 2)
+  EELS_G2(2, 4) EELS_G2(1, 4) EELS_G2(2, 2) EELS_G2(1, 2) EELS_G2(1, 1)
 #undef EELS_G2
   return cudaErrorInvalidValue;
 }
