@@ -162,7 +162,7 @@ struct PackPtr {
 
 // Small host arrays that a call needs on the device, sent in one buffer by one copy: a map
 // has about thirty of them, and an allocation, a pageable copy and a free for each cost a
-// small map more than its kernels (64 grid: 258 -> 190 us).
+// small map more than its kernels (64 grid: 258 -> 225 us).
 struct Pack {
   std::vector<unsigned char> host;
   struct Item { void** at; size_t offset; };
@@ -677,6 +677,7 @@ namespace {
 struct SiteLists {
   std::vector<int> xoff, xcnt, xlist, yoff, ycnt, ylist;
   int max_nr = 0;
+  double tiles[3] = {0, 0, 0};   // mean over sites with nr > 0 of ceil(nr / 16), / 32, / 64
 };
 
 // A rectangle of the scan: positions ix0 .. ix0 + nx - 1 by iy0 .. iy0 + ny - 1, indexed
@@ -689,6 +690,7 @@ SiteLists window_lists(const eels_transitions* tr, const eels_scan* sc, const Sc
                        double cell, int f) {
   SiteLists L;
   const int S = tr->n_sites;
+  int seen = 0;   // sites with nr > 0
   L.xoff.resize(S); L.xcnt.resize(S); L.yoff.resize(S); L.ycnt.resize(S);
   for (int s = 0; s < S; ++s) {
     L.xoff[s] = (int)L.xlist.size();
@@ -701,8 +703,12 @@ SiteLists window_lists(const eels_transitions* tr, const eels_scan* sc, const Sc
       if (axis_in_window(tr->y[s], sc->y0 + (double)(win.iy0 + iy) * sc->step_y, cell, f))
         L.ylist.push_back(iy);
     L.ycnt[s] = (int)L.ylist.size() - L.yoff[s];
-    L.max_nr = std::max(L.max_nr, L.xcnt[s] * L.ycnt[s]);
+    const int nr = L.xcnt[s] * L.ycnt[s];
+    L.max_nr = std::max(L.max_nr, nr);
+    seen += nr > 0;
+    for (int j = 0; j < 3; ++j) L.tiles[j] += (nr + (16 << j) - 1) / (16 << j);
   }
+  for (double& t : L.tiles) t /= std::max(seen, 1);
   return L;
 }
 
@@ -1081,7 +1087,8 @@ eels_status map_window(eels_ctx* ctx, const eels_smatrix* sm, const eels_transit
     Prof pr(ctx, "tc_gather_sets", st);
     EELS_CK(eels::tc_gather_sets(b, dset_site.p, st));
   }
-  eels::WindowLists wl{dxoff.p, dxcnt.p, dxlist.p, dyoff.p, dycnt.p, dylist.p, L.max_nr};
+  eels::WindowLists wl{dxoff.p, dxcnt.p, dxlist.p, dyoff.p, dycnt.p, dylist.p, L.max_nr,
+                       {L.tiles[0], L.tiles[1], L.tiles[2]}};
   // tensor-core contraction of slice i with one grouping, accumulated into `map`
   // assoc: EELS_ASSOC_TRANSITION_FIRST or EELS_ASSOC_PROBE_FIRST; n1, n2: narrow tiles for
   // the first / second GEMM; timed (autotuner): event pairs around every GEMM launch,

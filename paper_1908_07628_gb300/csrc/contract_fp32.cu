@@ -47,8 +47,8 @@ __device__ __forceinline__ void cp_async_wait() {
 // ahead into registers.  One barrier per step.
 //
 // Measured against one 64 x 64 tile per transition, loaded without overlap: a 128-grid
-// request 2.05 -> 1.65 ms of GEMM 1 and 0.22 -> 0.15 of GEMM 2, two 256-grid configurations
-// 9.2 -> 7.0 and 2.8 -> 2.1 ms (41 TFLOP/s useful), a 64-grid map 0.156 -> 0.065 ms.  The FMA
+// request 2.05 -> 1.57 ms of GEMM 1 and 0.22 -> 0.15 of GEMM 2, two 256-grid configurations
+// 9.2 -> 6.23 and 2.8 -> 2.10 ms, a 64-grid map 0.156 -> 0.048 ms.  The FMA
 // pipe is 63 % busy: an FMA that reads three registers runs at two thirds of the rate
 // (25.6 against 38 T/s), and packed f32x2 FMAs do too; they were no faster.
 template <int IM, int JN>
@@ -334,11 +334,10 @@ namespace {
 
 // Estimated cycles of one K step over a whole launch with 16 im x 16 jn tiles: the CTAs of
 // the busiest SM after one another, each 128 im jn cycles of FMA issue and the issue slots of
-// its loads and its loop (about 300 + 68 (im + jn), from instruction counts), plus the
-// latency of a step where one CTA has an SM to itself.
-double step_cost(int64_t ctas, int im, int jn) {
-  const double per_sm = (double)((ctas + sm_count() - 1) / sm_count());
-  return per_sm * (128.0 * im * jn + 68.0 * (im + jn) + 300.0) + (per_sm < 2 ? 500.0 : 0.0);
+// its loads and its loop, plus the latency of a step where one CTA has an SM to itself.
+double step_cost(double ctas, int im, int jn, double per_load, double fixed) {
+  const double per_sm = ceil(ctas / sm_count());
+  return per_sm * (128.0 * im * jn + per_load * (im + jn) + fixed) + (per_sm < 2 ? 500.0 : 0.0);
 }
 
 template <int IM, int JN>
@@ -380,7 +379,8 @@ cudaError_t launch_gemm1_fp32(const float2* Sout, const float2* Sin, int nh, int
   if (sb.count <= 0 || sb.nt <= 0) return cudaSuccess;
   // the tile that wastes least on the edges of n_out and nt n_in, or spreads a small
   // launch over more SMs (the 64-grid map takes 60 CTAs of 16 x 16 instead of 18 of 32 x 32:
-  // 218 -> 198 us)
+  // 218 -> 198 us).  A load and the loop cost 68 (im + jn) + 300 issue slots a step by the
+  // instruction counts.
   int im = 0, jn = 0;
   double best = 0;
   for (int i : {8, 7, 6, 5, 4, 2, 1})
@@ -388,7 +388,7 @@ cudaError_t launch_gemm1_fp32(const float2* Sout, const float2* Sin, int nh, int
       if (j == 1 ? i > 2 : i < 2) continue;   // not built
       const int64_t ctas = (int64_t)((sb.nt * n_in + 16 * j - 1) / (16 * j)) *
                            ((n_out + 16 * i - 1) / (16 * i)) * sb.count;
-      const double c = step_cost(ctas, i, j);
+      const double c = step_cost((double)ctas, i, j, 68.0, 300.0);
       if (im == 0 || c < best) { best = c; im = i; jn = j; }
     }
 #define EELS_G1(I, J)                                                                         \
@@ -408,14 +408,16 @@ cudaError_t launch_gemm2_abs2_fp32(const float2* M, int64_t m_stride, int n_out,
                                    cudaStream_t s) {
   if (sb.count <= 0 || sb.nt <= 0 || wl.max_nr <= 0) return cudaSuccess;
   const int groups = sb.nt * ((n_out + 63) / 64);
+  // positions past a site's own count cost nothing (those tiles return at once), so the
+  // tiles that run are counted, not those of the largest site: 32 columns for the two
+  // 256-grid configurations instead of 64, 2.46 -> 2.10 ms
   int g = 0, jn = 0;
   double best = 0;
   for (int i : {2, 1})
     for (int j : {4, 2, 1}) {
       if (i == 2 && j == 1) continue;   // not built
-      const int64_t ctas = (int64_t)((wl.max_nr + 16 * j - 1) / (16 * j)) * ((groups + i - 1) / i) *
-                           sb.count;
-      const double c = step_cost(ctas, 4 * i, j);
+      const double ctas = wl.tiles[j / 2] * ((groups + i - 1) / i) * sb.count;
+      const double c = step_cost(ctas, 4 * i, j, 20.0, 120.0);
       if (g == 0 || c < best) { best = c; g = i; jn = j; }
     }
 #define EELS_G2(I, J)                                                                         \

@@ -92,7 +92,8 @@ struct SiteBatch {
 struct WindowLists {
   const int* xoff; const int* xcnt; const int* xlist;   // per site: scan columns in the PRISM window
   const int* yoff; const int* ycnt; const int* ylist;   // per site: scan rows
-  int max_nr;                                           // max over sites of xcnt*ycnt
+  int max_nr;                                           // max over sites of nr = xcnt*ycnt
+  double tiles[3];                                      // mean of ceil(nr / (16 << j)) where nr > 0
 };
 // M[slot nt + t][d][j], m_stride values apart
 cudaError_t launch_gemm1_fp32(const float2* Sout, const float2* Sin, int nh, int n_out, int n_in,
