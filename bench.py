@@ -389,7 +389,8 @@ def s2_study(g, ctx, stream, thickness_cells=(5, 12, 19, 23), reps=2):
 
 def _source_hash(kernel):
     import hashlib
-    files = (["paper_1908_07628_gb300/csrc/multislice.cu", "paper_1908_07628_gb300/csrc/common.cuh"]
+    files = (["paper_1908_07628_gb300/csrc/multislice.cu", "paper_1908_07628_gb300/csrc/plan_fft.cuh",
+              "paper_1908_07628_gb300/csrc/common.cuh"]
              if "pass" in kernel else
              ["paper_1908_07628_gb300/csrc/contract_tc.cu", "paper_1908_07628_gb300/csrc/tc_ptx.cuh"])
     m = hashlib.sha1()
