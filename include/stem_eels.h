@@ -114,8 +114,9 @@ typedef struct {
   double x0, y0, step_x, step_y;
 } eels_scan;
 
-/* Create a context on CUDA device `device`.  Owns twiddle tables, options, the grouping
- * choices of the autotuner and the profiling records.  A context serves one host thread
+/* Create a context on CUDA device `device`.  Owns twiddle tables (a map server's are
+ * shared by the contexts of its requests), options, the grouping choices of the autotuner
+ * and the profiling records.  A context serves one host thread
  * at a time; threads that compute concurrently each use their own context (as the map
  * server's workers do).  Different contexts may run concurrently on one device. */
 eels_status eels_create(int device, eels_ctx** out);

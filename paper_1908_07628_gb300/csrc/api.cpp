@@ -12,6 +12,7 @@
 #include <cstdio>
 #include <cstring>
 #include <map>
+#include <memory>
 #include <mutex>
 #include <string>
 #include <unordered_map>
@@ -46,6 +47,7 @@ struct eels_ctx {
   struct Choice { int assoc; int narrow1, narrow2; };
   std::map<std::vector<int64_t>, Choice> assoc_cache;
   std::string err;
+  std::shared_ptr<eels::TwiddleTables> tables;   // its own, or those of the server it works for
   // kernel timing records (eels_profile_enable)
   bool profiling = false;
   struct Rec { const char* name; cudaEvent_t a, b; };
@@ -247,37 +249,8 @@ bool axis_in_window(double s, double r, double cell, int f) {
   return d >= -h && d < h;
 }
 
-// Twiddle tables exp(-2 pi i k/N) of a device, shared by its contexts (a map server makes
-// one context per request) and freed with the last of them: at most one table per grid and
-// cut size.  Uploaded with a synchronous copy, so any stream may read them afterwards.
-struct TwiddlePool {
-  int contexts = 0;
-  std::map<int, float2*> tables;
-};
-std::mutex g_twiddle_mu;
-// by device; never destroyed, so that a context may be destroyed at any time during exit
-std::map<int, TwiddlePool>& g_twiddles = *new std::map<int, TwiddlePool>();
-
 eels_status twiddles(eels_ctx* ctx, int n, float2** out) {
-  std::lock_guard<std::mutex> lock(g_twiddle_mu);
-  auto& tables = g_twiddles[ctx->device].tables;
-  auto it = tables.find(n);
-  if (it != tables.end()) {
-    *out = it->second;
-    return EELS_OK;
-  }
-  const int len = eels::twiddle_table_size(n);
-  std::vector<float2> h(len);
-  eels::fill_twiddle_tables(n, h.data());
-  float2* d = nullptr;
-  EELS_CK(cudaMalloc((void**)&d, len * sizeof(float2)));
-  const cudaError_t e = cudaMemcpy(d, h.data(), len * sizeof(float2), cudaMemcpyHostToDevice);
-  if (e != cudaSuccess) {
-    cudaFree(d);
-    return cuda_fail(ctx, e, "twiddle table");
-  }
-  tables[n] = d;
-  *out = d;
+  EELS_CK(ctx->tables->get(n, out));
   return EELS_OK;
 }
 
@@ -322,9 +295,41 @@ void eels::set_tile_hook(eels_ctx* ctx, TileHook fn, void* user) {
 
 double eels::last_map_flops(const eels_ctx* ctx) { return ctx ? ctx->last_map_flops : 0.0; }
 
-extern "C" {
+eels::TwiddleTables::~TwiddleTables() {
+  int current = 0;
+  const bool known = cudaGetDevice(&current) == cudaSuccess;
+  cudaSetDevice(device_);
+  for (auto& kv : by_size_) cudaFree(kv.second);
+  if (known) cudaSetDevice(current);
+  (void)cudaGetLastError();
+}
 
-eels_status eels_create(int device, eels_ctx** out) {
+cudaError_t eels::TwiddleTables::get(int n, float2** out) {
+  std::lock_guard<std::mutex> lock(mu_);
+  auto it = by_size_.find(n);
+  if (it == by_size_.end()) {
+    const int len = eels::twiddle_table_size(n);
+    std::vector<float2> h(len);
+    eels::fill_twiddle_tables(n, h.data());
+    float2* d = nullptr;
+    cudaError_t e = cudaMalloc((void**)&d, len * sizeof(float2));
+    if (e != cudaSuccess) return e;
+    // A copy from pageable memory may return before its bytes are on the device, and the
+    // streams that read the table need not be ordered after the copy's stream.
+    if ((e = cudaMemcpy(d, h.data(), len * sizeof(float2), cudaMemcpyHostToDevice)) !=
+            cudaSuccess ||
+        (e = cudaStreamSynchronize(cudaStreamLegacy)) != cudaSuccess) {
+      cudaFree(d);
+      return e;
+    }
+    it = by_size_.emplace(n, d).first;
+  }
+  *out = it->second;
+  return cudaSuccess;
+}
+
+eels_status eels::create_context(int device, std::shared_ptr<TwiddleTables> tables,
+                                 eels_ctx** out) {
   if (!out) return EELS_ERR_ARG;
   *out = nullptr;
   int count = 0;
@@ -333,10 +338,7 @@ eels_status eels_create(int device, eels_ctx** out) {
   if (cudaSetDevice(device) != cudaSuccess) return EELS_ERR_CUDA;
   eels_ctx* c = new eels_ctx();
   c->device = device;
-  {
-    std::lock_guard<std::mutex> lock(g_twiddle_mu);
-    g_twiddles[device].contexts++;
-  }
+  c->tables = tables ? std::move(tables) : std::make_shared<TwiddleTables>(device);
   // keep freed stream-ordered allocations cached between calls
   cudaMemPool_t pool;
   if (cudaDeviceGetDefaultMemPool(&pool, device) == cudaSuccess) {
@@ -347,17 +349,15 @@ eels_status eels_create(int device, eels_ctx** out) {
   return EELS_OK;
 }
 
+extern "C" {
+
+eels_status eels_create(int device, eels_ctx** out) {
+  return eels::create_context(device, nullptr, out);
+}
+
 void eels_destroy(eels_ctx* ctx) {
   if (!ctx) return;
   cudaSetDevice(ctx->device);
-  {
-    std::lock_guard<std::mutex> lock(g_twiddle_mu);
-    TwiddlePool& pool = g_twiddles[ctx->device];
-    if (--pool.contexts == 0) {
-      for (auto& kv : pool.tables) cudaFree(kv.second);
-      pool.tables.clear();
-    }
-  }
   for (auto& r : ctx->recs) { cudaEventDestroy(r.a); cudaEventDestroy(r.b); }
   for (auto e : ctx->spare) cudaEventDestroy(e);
   delete ctx;

@@ -5,7 +5,11 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
-struct eels_ctx;
+#include <map>
+#include <memory>
+#include <mutex>
+
+#include "stem_eels.h"
 
 namespace eels {
 
@@ -17,6 +21,26 @@ typedef int (*TileHook)(void* user, int phase, int done, int total);
 void set_tile_hook(eels_ctx* ctx, TileHook fn, void* user);
 // Flops of the context's last map contraction as grouped (8 per complex product).
 double last_map_flops(const eels_ctx* ctx);
+
+// Device twiddle tables by transform length (fill_twiddle_tables), made when first asked for
+// and freed with the object.  A context has its own; the contexts of a map server, one per
+// request, share the server's.  Any thread may ask, with the device current.
+class TwiddleTables {
+ public:
+  explicit TwiddleTables(int device) : device_(device) {}
+  ~TwiddleTables();
+  TwiddleTables(const TwiddleTables&) = delete;
+  TwiddleTables& operator=(const TwiddleTables&) = delete;
+  // the table of length n, complete on the device: any stream may read it
+  cudaError_t get(int n, float2** out);
+
+ private:
+  const int device_;
+  std::mutex mu_;
+  std::map<int, float2*> by_size_;
+};
+// eels_create for a context that uses `tables` (null: its own).
+eels_status create_context(int device, std::shared_ptr<TwiddleTables> tables, eels_ctx** out);
 
 // True if the multislice kernels are compiled for grid side n.
 bool grid_supported(int n);

@@ -23,6 +23,7 @@
 #include <cstring>
 #include <deque>
 #include <map>
+#include <memory>
 #include <mutex>
 #include <string>
 #include <thread>
@@ -83,7 +84,7 @@ struct eels_server {
   int running = 0;                  // admitted requests not yet finished
   bool stop = false;
   double t0 = 0, t_first = -1, t_last = 0;
-  eels_ctx* base = nullptr;         // keeps the device's shared tables between requests
+  std::shared_ptr<eels::TwiddleTables> tables;   // of all requests' contexts
   std::thread admitter;
   std::vector<std::thread> threads;
 };
@@ -136,7 +137,7 @@ int tile_gate(void* user, int /*phase*/, int done, int total) {
 void run_request(eels_server* sv, Request* r) {
   cudaSetDevice(sv->device);
   eels_ctx* ctx = nullptr;
-  eels_status s = eels_create(sv->device, &ctx);
+  eels_status s = eels::create_context(sv->device, sv->tables, &ctx);
   if (s == EELS_OK && cudaStreamCreateWithFlags(&r->st, cudaStreamNonBlocking) != cudaSuccess)
     s = EELS_ERR_CUDA;
   if (s == EELS_OK) {
@@ -248,12 +249,8 @@ eels_status eels_server_create(int device, int64_t hbm_budget, int slots, eels_s
   if (cudaGetDeviceCount(&count) != cudaSuccess || device < 0 || device >= count)
     return EELS_ERR_CUDA;
   eels_server* sv = new eels_server();
-  const eels_status made = eels_create(device, &sv->base);
-  if (made != EELS_OK) {
-    delete sv;
-    return made;
-  }
   sv->device = device;
+  sv->tables = std::make_shared<eels::TwiddleTables>(device);
   sv->budget = hbm_budget;
   sv->slots = slots;
   sv->tokens = slots;
@@ -425,7 +422,6 @@ void eels_server_destroy(eels_server* sv) {
   // admitted requests run to completion; the admitter has stopped adding threads
   for (auto& t : sv->threads) t.join();
   for (auto& kv : sv->requests) delete kv.second;
-  eels_destroy(sv->base);
   delete sv;
 }
 
