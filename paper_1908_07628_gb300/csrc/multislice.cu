@@ -49,6 +49,98 @@ struct RowSmem {
                                   (size_t)pf::SetPart<N>::BOTH * sizeof(float2);
 };
 
+// Inputs of the inverse x-FFT of rows y0 .. y0 + SEQ - 1 of a wave: the band box, zero-padded
+// to N.  START: the wave is a plane wave, formed here instead of being read (the first slice
+// of a sweep; writing plane waves out and reading them back costs a build 4 % of its time).
+template <int N, bool START>
+__device__ __forceinline__ void row_load(float2* v, const float2* __restrict__ W,
+                                         const PlaneWaves& start, const float2* __restrict__ tw,
+                                         int64_t wave, int y0, int lane) {
+  constexpr int NH = N / 2, NQ = N / 4, SEQ = pf::Seqs<N>::SEQ;
+  using PI = pf::Plan2<N, true>;
+  int col = -1, ky = 0;   // START: the wave's box column (-1: none) and y frequency
+  float2 a = make_float2(0.f, 0.f);
+  if constexpr (START) {
+    const int p = start.px[wave];
+    if (STEM_REQUIRE(p >= -NH && p < NH)) col = p >= 0 ? p : p + NH;
+    ky = start.py[wave];
+    a = start.amp[wave];
+  }
+#pragma unroll
+  for (int t = 0; t < PI::PER0; ++t) {
+    const int u = lane + 32 * t;
+    if ((SEQ * PI::NB0) % 32 == 0 || u < SEQ * PI::NB0) {
+      const int y = y0 + u / PI::NB0, b = u % PI::NB0;
+      const float2* src = W + (wave * N + y) * NH + b;
+      float2 on = make_float2(0.f, 0.f);
+      if constexpr (START) {
+        const int m = ky * y % N;
+        on = cmul(a, cconj(__ldg(tw + (m < 0 ? m + N : m))));   // exp(+2 pi i ky y / N)
+      }
+#pragma unroll
+      for (int q = 0; q < PI::R0; ++q) {
+        const int at = q * PI::NB0;
+        float2 x = make_float2(0.f, 0.f);
+        if (at < NQ || at >= N - NQ) {
+          const int i = at < NQ ? at : at - NH;
+          if constexpr (START) x = b + i == col ? on : x;
+          else x = src[i];
+        }
+        v[t * PI::R0 + q] = x;
+      }
+    }
+  }
+}
+
+// The row pass of one wave's rows y0 .. y0 + SEQ - 1, loaded in v (row_load), by one warp:
+// trows holds their SEQ rows of t, fset and rset the factor sets of the two plans.
+template <int N, bool CONJ>
+__device__ __forceinline__ void row_wave(float2* v, float2* sbuf, const float2* trows,
+                                         const float2* fset, const float2* rset, int64_t wave,
+                                         int y0, int lane, float2* __restrict__ Phi,
+                                         int store_mode, float2* __restrict__ S, int s_waves,
+                                         int64_t s_stride, int fft_out) {
+  constexpr int NH = N / 2, NQ = N / 4;
+  constexpr int SEQ = pf::Seqs<N>::SEQ, LD = pf::Seqs<N>::PADDED;
+  using PF = pf::Plan2<N, false>;   // forward transform
+  pf::warp_fft<N, true, true, true>(v, sbuf, LD, rset, lane);
+
+  // real space: slot u holds N psi(x = u % NB0 + q N/R0, y0 + u / NB0)
+#pragma unroll
+  for (int t = 0; t < PF::PER0; ++t) {
+    const int u = lane + 32 * t;
+    if ((SEQ * PF::NB0) % 32 == 0 || u < SEQ * PF::NB0) {
+      const int y = y0 + u / PF::NB0, b = u % PF::NB0;
+      const float2* trow = trows + (u / PF::NB0) * N + b;
+      // even x only: N/R0 is even, so x has the parity of b
+      const bool store = store_mode != 0 && ((y | b) & 1) == 0 && wave < s_waves;
+      float2* srow = S + wave * s_stride + (int64_t)(y >> 1) * NH + (b >> 1);
+#pragma unroll
+      for (int q = 0; q < PF::R0; ++q) {
+        const float2 before = v[t * PF::R0 + q];
+        const float2 after = pf::mul_c<CONJ>(before, trow[q * PF::NB0]);
+        if (store) srow[q * (PF::NB0 / 2)] = store_mode == 1 ? after : before;
+        v[t * PF::R0 + q] = after;
+      }
+    }
+  }
+  if (!fft_out) return;
+  pf::warp_fft<N, false, false, false>(v, sbuf, LD, fset, lane);
+#pragma unroll
+  for (int t = 0; t < PF::PER1; ++t) {
+    const int u = lane + 32 * t;
+    if ((SEQ * PF::NB1) % 32 == 0 || u < SEQ * PF::NB1) {
+      float2* dst = Phi + (wave * N + y0) * NH + (u / PF::NB1) * NH + u % PF::NB1;
+#pragma unroll
+      for (int q = 0; q < PF::R1; ++q) {
+        const int at = q * PF::NB1;
+        if (at < NQ) dst[at] = v[t * PF::R1 + q];
+        else if (at >= N - NQ) dst[at - NH] = v[t * PF::R1 + q];
+      }
+    }
+  }
+}
+
 // Row pass.  A CTA takes SEQ rows y0 .. y0 + SEQ - 1 of `chunk` waves, one warp a wave at a
 // time: the rows of t and the factor sets lie in shared memory for all of them (read per
 // row from L2 and L1 they cost as many wavefronts and far more latency), and the rows of a
@@ -56,18 +148,13 @@ struct RowSmem {
 // (ncu, 1024: 69 %, FMA pipe 55 %, shared-memory wavefronts 66 %, DRAM 45 %).  Adjoint pass
 // with the S_out store, us per wave, before -> now: 1024: 3.22 -> 2.95, 768: 1.83 -> 1.55,
 // 512: 0.58 -> 0.57, 384: 1.00 -> 0.48 (four stages and three exchanges before).
-// START: the waves are plane waves, formed here instead of being read (the first slice of a
-// sweep; writing them out and reading them back cost a build 4 % of its time).
 template <int N, bool CONJ, bool START>
 __global__ void __launch_bounds__(kRowWarps * 32, row_ctas<N>())
 k_row_pass(const float2* __restrict__ W, const PlaneWaves start, float2* __restrict__ Phi,
            const float2* __restrict__ t_slice, int store_mode, float2* __restrict__ S,
            int s_waves, int64_t s_stride, int fft_out, const float2* __restrict__ tw,
            int n_waves, int chunk) {
-  constexpr int NH = N / 2, NQ = N / 4;
-  constexpr int SEQ = pf::Seqs<N>::SEQ, LD = pf::Seqs<N>::PADDED;
-  using PI = pf::Plan2<N, true>;    // inverse transform: reversed radix plan
-  using PF = pf::Plan2<N, false>;   // forward transform
+  constexpr int NH = N / 2, SEQ = pf::Seqs<N>::SEQ;
   extern __shared__ float2 smem[];
   float2* trows = smem + kRowWarps * RowSmem<N>::BUF;   // [SEQ][N]
   float2* sets = trows + SEQ * N;
@@ -79,90 +166,59 @@ k_row_pass(const float2* __restrict__ W, const PlaneWaves start, float2* __restr
   pf::copy_async(trows, t_slice + (int64_t)y0 * N, SEQ * N);
 
   float2 v[pf::Seqs<N>::E];
-  // inputs of the inverse x-FFT: the band box, zero-padded to N
-  auto load = [&](int64_t wave) {
-    int col = -1, ky = 0;   // START: the wave's box column (-1: none) and y frequency
-    float2 a = make_float2(0.f, 0.f);
-    if constexpr (START) {
-      const int p = start.px[wave];
-      if (STEM_REQUIRE(p >= -NH && p < NH)) col = p >= 0 ? p : p + NH;
-      ky = start.py[wave];
-      a = start.amp[wave];
-    }
-#pragma unroll
-    for (int t = 0; t < PI::PER0; ++t) {
-      const int u = lane + 32 * t;
-      if ((SEQ * PI::NB0) % 32 == 0 || u < SEQ * PI::NB0) {
-        const int y = y0 + u / PI::NB0, b = u % PI::NB0;
-        const float2* src = W + (wave * N + y) * NH + b;
-        float2 on = make_float2(0.f, 0.f);
-        if constexpr (START) {
-          const int m = ky * y % N;
-          on = cmul(a, cconj(__ldg(tw + (m < 0 ? m + N : m))));   // exp(+2 pi i ky y / N)
-        }
-#pragma unroll
-        for (int q = 0; q < PI::R0; ++q) {
-          const int at = q * PI::NB0;
-          float2 x = make_float2(0.f, 0.f);
-          if (at < NQ || at >= N - NQ) {
-            const int i = at < NQ ? at : at - NH;
-            if constexpr (START) x = b + i == col ? on : x;
-            else x = src[i];
-          }
-          v[t * PI::R0 + q] = x;
-        }
-      }
-    }
-  };
-  if (w0 < w_end) load(w0);
+  if (w0 < w_end) row_load<N, START>(v, W, start, tw, w0, y0, lane);
   pf::cp_async_wait();
   __syncthreads();
 
   for (int64_t wave = w0; wave < w_end; wave += kRowWarps) {
-    const int64_t base = (wave * N + y0) * NH;
-    if (wave != w0) load(wave);
+    if (wave != w0) row_load<N, START>(v, W, start, tw, wave, y0, lane);
     if (!START && wave + kRowWarps < w_end) {   // the next rows: SEQ * NH values, contiguous
-      const float2* next = W + base + (int64_t)kRowWarps * N * NH;
+      const float2* next = W + ((wave + kRowWarps) * N + y0) * NH;
 #pragma unroll
       for (int i = lane * 16; i < SEQ * NH; i += 512) prefetch_l2(next + i);
     }
-    pf::warp_fft<N, true, true, true>(v, sbuf, LD, pf::rev_set<N>(sets), lane);
-
-    // real space: slot u holds N psi(x = u % NB0 + q N/R0, y0 + u / NB0)
-#pragma unroll
-    for (int t = 0; t < PF::PER0; ++t) {
-      const int u = lane + 32 * t;
-      if ((SEQ * PF::NB0) % 32 == 0 || u < SEQ * PF::NB0) {
-        const int y = y0 + u / PF::NB0, b = u % PF::NB0;
-        const float2* trow = trows + (u / PF::NB0) * N + b;
-        // even x only: N/R0 is even, so x has the parity of b
-        const bool store = store_mode != 0 && ((y | b) & 1) == 0 && wave < s_waves;
-        float2* srow = S + wave * s_stride + (int64_t)(y >> 1) * NH + (b >> 1);
-#pragma unroll
-        for (int q = 0; q < PF::R0; ++q) {
-          const float2 before = v[t * PF::R0 + q];
-          const float2 after = pf::mul_c<CONJ>(before, trow[q * PF::NB0]);
-          if (store) srow[q * (PF::NB0 / 2)] = store_mode == 1 ? after : before;
-          v[t * PF::R0 + q] = after;
-        }
-      }
-    }
-    if (!fft_out) continue;
-    pf::warp_fft<N, false, false, false>(v, sbuf, LD, sets, lane);
-#pragma unroll
-    for (int t = 0; t < PF::PER1; ++t) {
-      const int u = lane + 32 * t;
-      if ((SEQ * PF::NB1) % 32 == 0 || u < SEQ * PF::NB1) {
-        float2* dst = Phi + base + (u / PF::NB1) * NH + u % PF::NB1;
-#pragma unroll
-        for (int q = 0; q < PF::R1; ++q) {
-          const int at = q * PF::NB1;
-          if (at < NQ) dst[at] = v[t * PF::R1 + q];
-          else if (at >= N - NQ) dst[at - NH] = v[t * PF::R1 + q];
-        }
-      }
-    }
+    row_wave<N, CONJ>(v, sbuf, trows, sets, pf::rev_set<N>(sets), wave, y0, lane, Phi, store_mode,
+                      S, s_waves, s_stride, fft_out);
   }
+}
+
+// Row pass of few waves: a warp takes SEQ rows of one wave and the CTA's warps neighbouring
+// rows; t and the factor sets are read where they lie (L2, L1) and no warp waits for another.
+// Where a warp has one or two waves, k_row_pass spends as long on filling shared memory as
+// on a wave, and of the 4 m + 1 beams of an aperture three warps of the last CTA have none.
+// Mean row launch of a build, us, k_row_pass -> this: 512: 9 waves 16.2 -> 12.4, 37 34.7 ->
+// 30.5; 256: 37 13.9 -> 12.3; 1024: 5 28.3 -> 24.5; 768: 9 28.4 -> 23.8; 128: 37 8.3 -> 8.2.
+// Six CTAs per SM at 256 (80 registers): 145 waves 28.5 us, with five 30.0.
+template <int N>
+__host__ __device__ constexpr int few_ctas() {
+  return N == 256 ? 6 : row_ctas<N>();
+}
+template <int N>
+__global__ void __launch_bounds__(kRowWarps * 32, few_ctas<N>())
+k_row_pass_few(const float2* __restrict__ W, const PlaneWaves start, float2* __restrict__ Phi,
+               const float2* __restrict__ t_slice, int conj_t, int store_mode,
+               float2* __restrict__ S, int s_waves, int64_t s_stride, int fft_out,
+               const float2* __restrict__ tw) {
+  constexpr int SEQ = pf::Seqs<N>::SEQ;
+  extern __shared__ float2 smem[];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  float2* sbuf = smem + warp * RowSmem<N>::BUF;
+  const int y0 = (blockIdx.x * kRowWarps + warp) * SEQ;
+  const int64_t wave = blockIdx.y;
+  const float2* fset = tw + pf::set_offset(N, false, false) + pf::SetPart<N>::FROM;
+  const float2* rset = pf::SetPart<N>::SAME
+                           ? fset
+                           : tw + pf::set_offset(N, false, true) + pf::SetPart<N>::FROM;
+  const float2* trows = t_slice + (int64_t)y0 * N;
+  float2 v[pf::Seqs<N>::E];
+  if (start.px) row_load<N, true>(v, W, start, tw, wave, y0, lane);
+  else row_load<N, false>(v, W, start, tw, wave, y0, lane);
+  if (conj_t)
+    row_wave<N, true>(v, sbuf, trows, fset, rset, wave, y0, lane, Phi, store_mode, S, s_waves,
+                      s_stride, fft_out);
+  else
+    row_wave<N, false>(v, sbuf, trows, fset, rset, wave, y0, lane, Phi, store_mode, S, s_waves,
+                       s_stride, fft_out);
 }
 
 // Column pass.  A CTA takes CB neighbouring columns of `chunk` waves, a wave at a time; a
@@ -178,8 +234,8 @@ k_row_pass(const float2* __restrict__ W, const PlaneWaves start, float2* __restr
 template <int N>
 struct ColCfg {
   using PF = pf::Plan2<N, false>;
-  static constexpr int CB = N == 512 || N == 1024 ? 16 : 8;
-  static constexpr int CTAS = N == 64 ? 8 : N == 128 || N == 256 ? 5 : N == 384 ? 3 : N == 768 ? 2 : 1;
+  static constexpr int CB = N == 512 ? 16 : 8;
+  static constexpr int CTAS = N == 64 ? 8 : N == 128 || N == 256 ? 5 : N == 384 ? 3 : 2;
   static constexpr int TPC = pf::col_threads(N), THREADS = CB * TPC;
   static constexpr int PER0 = (PF::NB0 + TPC - 1) / TPC, PER1 = (PF::NB1 + TPC - 1) / TPC;
   static constexpr int E = PER0 * PF::R0 > PER1 * PF::R1 ? PER0 * PF::R0 : PER1 * PF::R1;
@@ -474,6 +530,11 @@ int wave_chunk(int n_waves, int blocks_x, int width, int resident) {
   return width * (int)std::min<int64_t>(per, 16);
 }
 
+// Launches of up to this many row groups (SEQ rows of a wave) go to k_row_pass_few, `warps` of
+// k_row_pass being resident on an SM.  Rounds of resident warps at which the two take the
+// same time: 64: 4, 128: 8, 256: 10, 512: 13, 768: 18, 1024: 11 to 20, 384: about 50.
+int64_t few_rows(int warps) { return 11LL * warps * sm_count(); }
+
 template <int N, bool CONJ, bool START>
 cudaError_t row_pass_c(int n_waves, const float2* W, const PlaneWaves& start, float2* Phi,
                        const float2* t, int store_mode, float2* S, int s_waves, int64_t s_stride,
@@ -494,6 +555,16 @@ cudaError_t row_pass_n(int n_waves, const float2* W, const PlaneWaves* start, fl
                        const float2* t, int conj_t, int store_mode, float2* S, int s_waves,
                        int64_t s_stride, int fft_out, const float2* tw, cudaStream_t s) {
   const PlaneWaves pw = start ? *start : PlaneWaves{};
+  if ((int64_t)n_waves * (N / pf::Seqs<N>::SEQ) <= few_rows(kRowWarps * row_ctas<N>())) {
+    static std::atomic<uint64_t> attr{0};
+    constexpr size_t smem = (size_t)kRowWarps * RowSmem<N>::BUF * sizeof(float2);
+    cudaError_t e = smem_attr_once(k_row_pass_few<N>, smem, attr);
+    if (e != cudaSuccess) return e;
+    dim3 grid(N / (kRowWarps * pf::Seqs<N>::SEQ), n_waves);
+    k_row_pass_few<N><<<grid, kRowWarps * 32, smem, s>>>(W, pw, Phi, t, conj_t, store_mode, S,
+                                                         s_waves, s_stride, fft_out, tw);
+    return cudaGetLastError();
+  }
   const auto fn = conj_t ? (start ? row_pass_c<N, true, true> : row_pass_c<N, true, false>)
                          : (start ? row_pass_c<N, false, true> : row_pass_c<N, false, false>);
   return fn(n_waves, W, pw, Phi, t, store_mode, S, s_waves, s_stride, fft_out, tw, s);
