@@ -4,7 +4,10 @@ Row pass: few waves take k_row_pass_few, many k_row_pass, whose warps then go th
 waves.  The whole build is past that line; the static build runs the same beams in groups
 that fit its 64 MiB, below it.  Both have the same bits, and the whole build is within 1e-5
 of the FP64 oracle per depth (the bound of the S-matrix parity test).  The conventional
-algorithm runs enough waves for the column pass with the detector sum to go through several."""
+algorithm runs enough waves for the column pass with the detector sum to go through several.
+
+Window gathers: a launch of few sites spreads a window over warps.  The map of the same sites
+in batches below and above that line differs by the order of the FP64 map sums (1e-12)."""
 import numpy as np
 import pytest
 
@@ -60,3 +63,23 @@ def test_many_waves_of_the_conventional_algorithm(g, n, scan_n, waves):
     want = lin.linear_map(wl)
     got = g.quadratic_reference_map_for(g.Context(0), wl)[0]
     assert np.linalg.norm(got - want) / np.linalg.norm(want) < 1e-4
+
+
+@pytest.mark.parametrize("prec", ["tf32", "bf16x3"])
+@pytest.mark.parametrize("w", [16, 17, 23, 32])   # 256, 289, 529 and 1024 window pixels
+def test_gathers_below_and_above_the_line(g, prec, w):
+    # 317 beams in, 349 or more out: 40 CTAs and more per site, the line at 16 per SM
+    wl = _workload(128, 10.0, n_sites=200, w=w, scan_n=3)
+    ctx = g.Context(0)
+    sm = g.build_smatrix_for(ctx, wl)
+    assert sm.n_in == 317
+    for how in ("transition_first", "probe_first"):
+        ctx.set_association(how)
+        ctx.set_tile_width(128)
+        ctx.set_batch_sites(0)
+        many = g.inelastic_map_for(ctx, sm, wl, prec)
+        ctx.set_batch_sites(5)
+        few = g.inelastic_map_for(ctx, sm, wl, prec)
+        assert np.linalg.norm(few - many) <= 1e-12 * np.linalg.norm(many), how
+    want = g.inelastic_map_for(ctx, sm, wl, "fp32")
+    assert np.linalg.norm(many - want) / np.linalg.norm(want) < 1e-3
