@@ -352,7 +352,8 @@ int eels_profile_read(eels_ctx* ctx, char* buf, int cap);
 /* The autotuner's choices kept in the context (EELS_ASSOC_AUTO): a JSON list with one
  * object per contraction shape {"precision", "n", "n_out", "n_in", "w", "nr_max",
  * "n_types", "grouping", "tile_first", "tile_second"} (tile widths of the grouping's
- * first and second GEMM).  Returns the bytes the text needs with its NUL; writes it if
+ * first and second GEMM).  Maps of equal sizes whose sites share their probe rows and maps
+ * whose sites do not are two shapes.  Returns the bytes the text needs with its NUL; writes it if
  * buf holds that many. */
 int eels_tuning_read(eels_ctx* ctx, char* buf, int cap);
 

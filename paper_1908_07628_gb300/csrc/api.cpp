@@ -899,8 +899,36 @@ eels_status map_window(eels_ctx* ctx, const eels_smatrix* sm, const eels_transit
   const int kal = eels::tc_k_align(tc_prec);
   const int k1p = (int)rup(2 * (int64_t)w * w, kal), k2p = (int)rup(2 * (int64_t)n_in, kal);
   const int nr_cap = std::max(L.max_nr, 1);
-  // AUTO: measured once per shape (both groupings timed on the first occupied slice)
-  const std::vector<int64_t> shape_key = {tc_prec, n, n_out, n_in, w, nr_cap, T};
+  const int vbytes = tc ? eels::tc_value_bytes(tc_prec) : 4;   // operand bytes per value
+  const int vf = vbytes / 4;                                      // ... in floats
+  // operand bytes with the buffers of either grouping (tr, pr) or both: probe rows of a set
+  // (AY, B2), and a site's other operands
+  const auto probe_bytes_of = [&](bool tr, bool pr) -> int64_t {
+    return vbytes * ((pr ? (int64_t)nr_cap * k2p : 0) + (tr ? (int64_t)2 * nr_cap * k2p : 0));
+  };
+  const auto site_bytes_of = [&](bool tr, bool pr) -> int64_t {
+    return vbytes * ((int64_t)n_out * k1p +
+                     (pr ? (int64_t)k1p * k2p + (int64_t)T * 2 * nr_cap * k1p : 0) +
+                     (tr ? (int64_t)T * 2 * n_in * k1p + (int64_t)T * n_out * k2p : 0));
+  };
+  // Probe rows do not depend on the depth: where at least every second site repeats the
+  // probes of another and the sets take at most a quarter of the operand budget, they are
+  // gathered once for the whole map, otherwise per site with each batch (the 80 A sphere:
+  // nearly every site has its own probes).  The number of sets, 0: per site.
+  ProbeSets sets;
+  if (tc) sets = probe_sets(L, slot_all);
+  const auto shared_sets = [&](bool tr, bool pr) -> int {
+    const int64_t u = (int64_t)sets.set_site.size(), bytes = u * probe_bytes_of(tr, pr);
+    const bool share = tc && 2 * u <= (int64_t)slot_all.size() && u <= 65535 &&
+                       4 * bytes <= ctx->operand_budget &&
+                       bytes + site_bytes_of(tr, pr) <= ctx->operand_budget;
+    return share ? (int)u : 0;
+  };
+  // AUTO: measured once per shape (both groupings timed on the first occupied slice).  The
+  // times hold the gathers of probe rows that are not shared, so maps that share them and
+  // maps that do not are different shapes.
+  const std::vector<int64_t> shape_key = {tc_prec, n, n_out, n_in, w, nr_cap, T,
+                                          shared_sets(true, true) > 0};
   int chosen = ctx->assoc;
   // complex products of each grouping over the map's sites (Eq. SHn0 applied to the probes)
   double c_tr = 0, c_pr = 0;
@@ -951,28 +979,9 @@ eels_status map_window(eels_ctx* ctx, const eels_smatrix* sm, const eels_transit
   bool tune = tc && chosen == EELS_ASSOC_AUTO;
   const bool need_tr = tune || chosen == EELS_ASSOC_TRANSITION_FIRST;
   const bool need_pr = tune || chosen == EELS_ASSOC_PROBE_FIRST;
-  const int vbytes = tc ? eels::tc_value_bytes(tc_prec) : 4;   // operand bytes per value
-  const int vf = vbytes / 4;                                      // ... in floats
-  // probe rows of a set (AY, B2), and a site's other operands
-  const int64_t probe_bytes = vbytes * ((need_pr ? (int64_t)nr_cap * k2p : 0) +
-                                        (need_tr ? (int64_t)2 * nr_cap * k2p : 0));
-  const int64_t site_bytes =
-      vbytes * ((int64_t)n_out * k1p +
-           (need_pr ? (int64_t)k1p * k2p + (int64_t)T * 2 * nr_cap * k1p : 0) +
-           (need_tr ? (int64_t)T * 2 * n_in * k1p + (int64_t)T * n_out * k2p : 0));
-  // Probe rows do not depend on the depth: where at least every second site repeats the
-  // probes of another and the sets take at most a quarter of the operand budget, they are
-  // gathered once for the whole map, otherwise per site with each batch (the 80 A sphere:
-  // nearly every site has its own probes).
-  ProbeSets sets;
-  int n_sets = 0;
-  if (tc) {
-    sets = probe_sets(L, slot_all);
-    const int64_t u = (int64_t)sets.set_site.size();
-    if (2 * u <= (int64_t)slot_all.size() && 4 * u * probe_bytes <= ctx->operand_budget &&
-        u * probe_bytes + site_bytes <= ctx->operand_budget && u <= 65535)
-      n_sets = (int)u;
-  }
+  const int64_t probe_bytes = probe_bytes_of(need_tr, need_pr);
+  const int64_t site_bytes = site_bytes_of(need_tr, need_pr);
+  const int n_sets = shared_sets(need_tr, need_pr);
   const int64_t per_site = site_bytes + (n_sets ? 0 : probe_bytes);
   int sb = (int)std::max<int64_t>(1, std::min<int64_t>(
       std::max(max_sites, 1), (ctx->operand_budget - n_sets * probe_bytes) / per_site));
