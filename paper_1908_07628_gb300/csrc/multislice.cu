@@ -225,17 +225,18 @@ k_row_pass_few(const float2* __restrict__ W, const PlaneWaves start, float2* __r
 // thread holds a butterfly of one column, and the lanes of a warp run over the columns
 // first, so that rows are read and written in segments of CB values straight from
 // registers and shared memory carries only the exchange inside each transform.  (One warp
-// per column with the tile staged in shared memory, the form before, took twice the
-// wavefronts and was bound by them.)  Measured, us per wave, before -> now: 1024: 2.41 ->
-// 1.91, 768: 1.69 -> 1.06, 512: 0.466 -> 0.387, 384: 0.66 -> 0.28, 256: 0.118 -> 0.106; the
-// copy bandwidth would allow 1.23, 0.69, 0.31, 0.17 and 0.08.  CB and CTAs per SM are the
-// fastest measured: 16 columns (128-byte segments) for the grids whose CTA then fills half
-// of an SM's warps by itself, 8 elsewhere.
-template <int N>
+// per column with the tile staged in shared memory took twice the wavefronts and was bound
+// by them.)  us per wave of a pass of many waves, with the staged tile / so: 1024: 2.18 /
+// 1.74, 768: 1.70 / 1.06, 512: 0.468 / 0.377, 384: 0.64 / 0.26, 256: 0.109 / 0.101; the copy
+// bandwidth would allow 1.23, 0.69, 0.31, 0.17 and 0.08.  CB (columns, col_pass_m) and CTAS
+// (CTAs per SM) are the fastest measured; at 768 and 1024 two CTAs of 8 columns are all the
+// registers that an SM has, 16 of its 64 warps.
+template <int N, int COLS>
 struct ColCfg {
   using PF = pf::Plan2<N, false>;
-  static constexpr int CB = N == 512 ? 16 : 8;
-  static constexpr int CTAS = N == 64 ? 8 : N == 128 || N == 256 ? 5 : N == 384 ? 3 : 2;
+  static constexpr int CB = COLS;
+  static constexpr int CTAS = N == 64 ? 8 : N == 128 || N == 256 ? 5 : N == 384 ? 3
+                            : N == 1024 && CB == 16 ? 1 : 2;
   static constexpr int TPC = pf::col_threads(N), THREADS = CB * TPC;
   static constexpr int PER0 = (PF::NB0 + TPC - 1) / TPC, PER1 = (PF::NB1 + TPC - 1) / TPC;
   static constexpr int E = PER0 * PF::R0 > PER1 * PF::R1 ? PER0 * PF::R0 : PER1 * PF::R1;
@@ -245,14 +246,14 @@ struct ColCfg {
 
 // MODE 0 / 1: multiply by the propagator table / its conjugate and go back to rows;
 // MODE 2: multiply by the table and sum |.|^2 over the detector bins.
-template <int N, int MODE>
-__global__ void __launch_bounds__(ColCfg<N>::THREADS, ColCfg<N>::CTAS)
+template <int N, int MODE, int CB>
+__global__ void __launch_bounds__(ColCfg<N, CB>::THREADS, ColCfg<N, CB>::CTAS)
 k_col_pass(const float2* __restrict__ Phi, float2* __restrict__ W, const float2* __restrict__ ptab,
            const uint8_t* __restrict__ det_mask, const int* __restrict__ wave_out,
            double* __restrict__ det_acc, double det_scale, const float2* __restrict__ tw,
            int n_waves, int chunk) {
-  using CC = ColCfg<N>;
-  constexpr int NH = N / 2, NQ = N / 4, CB = CC::CB;
+  using CC = ColCfg<N, CB>;
+  constexpr int NH = N / 2, NQ = N / 4;
   using PF = pf::Plan2<N, false>;
   using PI = pf::Plan2<N, true>;
   constexpr bool EXACT = pf::exact_factors(N, true);
@@ -530,6 +531,22 @@ int wave_chunk(int n_waves, int blocks_x, int width, int resident) {
   return width * (int)std::min<int64_t>(per, 16);
 }
 
+// The chunk between half and twice of `chunk` (at most 16) whose rounds of CTAs, two to an
+// SM, take least, the largest of equal ones.  A last round of at most one CTA per SM takes
+// about 0.6 of a full one.  512 columns pass: 593 waves in chunks of 10 leave a fourth round
+// of 48 CTAs, in chunks of 16 two full rounds.
+int even_rounds(int n_waves, int blocks_x, int chunk) {
+  const int64_t sms = sm_count();
+  int best = chunk;
+  double least = 0;
+  for (int c = std::min(2 * chunk, 16); 2 * c >= chunk && c > 0; --c) {
+    const int64_t ctas = (int64_t)((n_waves + c - 1) / c) * blocks_x, rest = ctas % (2 * sms);
+    const double time = c * (double(ctas / (2 * sms)) + (rest > sms ? 1.0 : rest ? 0.6 : 0.0));
+    if (least == 0 || time < least) { least = time; best = c; }
+  }
+  return best;
+}
+
 // Launches of up to this many row groups (SEQ rows of a wave) go to k_row_pass_few, `warps` of
 // k_row_pass being resident on an SM.  Rounds of resident warps at which the two take the
 // same time: 64: 4, 128: 8, 256: 10, 512: 13, 768: 18, 1024: 11 to 20, 384: about 50.
@@ -570,20 +587,36 @@ cudaError_t row_pass_n(int n_waves, const float2* W, const PlaneWaves* start, fl
   return fn(n_waves, W, pw, Phi, t, store_mode, S, s_waves, s_stride, fft_out, tw, s);
 }
 
+template <int N, int MODE, int CB>
+cudaError_t col_pass_c(int n_waves, const float2* Phi, float2* W, const float2* ptab,
+                       const uint8_t* det_mask, const int* wave_out, double* det_acc,
+                       double det_scale, const float2* tw, cudaStream_t s) {
+  using CC = ColCfg<N, CB>;
+  static std::atomic<uint64_t> attr{0};
+  cudaError_t e = smem_attr_once(k_col_pass<N, MODE, CB>, CC::BYTES, attr);
+  if (e != cudaSuccess) return e;
+  const int gx = N / 2 / CB;
+  int chunk = wave_chunk(n_waves, gx, 1, sm_count() * CC::CTAS);
+  if (CC::CTAS == 2) chunk = even_rounds(n_waves, gx, chunk);
+  dim3 grid(gx, (n_waves + chunk - 1) / chunk);
+  k_col_pass<N, MODE, CB><<<grid, CC::THREADS, CC::BYTES, s>>>(
+      Phi, W, ptab, det_mask, wave_out, det_acc, det_scale, tw, n_waves, chunk);
+  return cudaGetLastError();
+}
+
+// 16 columns (128-byte segments) at 512, and at 1024 for many waves: one CTA is then all that
+// an SM holds, and the last rounds weigh more than the longer segments give (1024, us a pass
+// with 8 and 16 columns: 317 waves 590 and 650, 1257 waves 2254 and 2237, 2801 waves 4999 and
+// 4881).
 template <int N, int MODE>
 cudaError_t col_pass_m(int n_waves, const float2* Phi, float2* W, const float2* ptab,
                        const uint8_t* det_mask, const int* wave_out, double* det_acc,
                        double det_scale, const float2* tw, cudaStream_t s) {
-  using CC = ColCfg<N>;
-  static std::atomic<uint64_t> attr{0};
-  cudaError_t e = smem_attr_once(k_col_pass<N, MODE>, CC::BYTES, attr);
-  if (e != cudaSuccess) return e;
-  const int gx = N / 2 / CC::CB;
-  const int chunk = wave_chunk(n_waves, gx, 1, sm_count() * CC::CTAS);
-  dim3 grid(gx, (n_waves + chunk - 1) / chunk);
-  k_col_pass<N, MODE><<<grid, CC::THREADS, CC::BYTES, s>>>(
-      Phi, W, ptab, det_mask, wave_out, det_acc, det_scale, tw, n_waves, chunk);
-  return cudaGetLastError();
+  const auto fn = [&] {
+    if constexpr (N == 1024) return n_waves < 1024 ? col_pass_c<N, MODE, 8> : col_pass_c<N, MODE, 16>;
+    else return col_pass_c<N, MODE, N == 512 ? 16 : 8>;
+  }();
+  return fn(n_waves, Phi, W, ptab, det_mask, wave_out, det_acc, det_scale, tw, s);
 }
 
 template <int N>
