@@ -1554,10 +1554,14 @@ eels_status eels_elastic_images(eels_ctx* ctx, const eels_smatrix* sm, const eel
                                    st, 1));
   EELS_CK(eels::launch_phase_table(ayT.p, dbq.p, n_in, f, sm->cell, sc->y0, sc->step_y, sc->n_sy,
                                    st, 1));
-  int max_span = 0;   // of the column origins of probes that one CTA may take together
+  // span of the column origins of probes that one CTA may take together, counted from the
+  // first of them or (a scan towards smaller x) from the last
+  int from_first = 0, from_last = 0;
   for (int i = 0; i < sc->n_sx; ++i)
-    for (int k = i; k < std::min(i + eels::kMaxCutProbes, sc->n_sx); ++k)
-      max_span = std::max(max_span, (wx[k] - wx[i] + nh) % nh);
+    for (int k = i; k < std::min(i + eels::kMaxCutProbes, sc->n_sx); ++k) {
+      from_first = std::max(from_first, (wx[k] - wx[i] + nh) % nh);
+      from_last = std::max(from_last, (wx[i] - wx[k] + nh) % nh);
+    }
   EELS_CK(dimg.alloc((size_t)n_det * n_img, st));
   EELS_CK(cudaMemsetAsync(dimg.p, 0, sizeof(double) * n_det * n_img, st));
   // scan rows in batches whose cuts fit in ~1 GiB
@@ -1569,7 +1573,8 @@ eels_status eels_elastic_images(eels_ctx* ctx, const eels_smatrix* sm, const eel
     {
       Prof pr(ctx, "exit_cut", st);
       EELS_CK(eels::launch_exit_cut(sm->s_exit, n_in, nh, m, axT.p, ayT.p, sc->n_sx, sc->n_sy,
-                                    dwx.p, dwy.p, iy0, nr, max_span, cuts.p, st));
+                                    dwx.p, dwy.p, iy0, nr, std::min(from_first, from_last),
+                                    from_last < from_first, cuts.p, st));
     }
     Prof pr(ctx, "cut_fft_detect", st);
     EELS_CK(eels::launch_cut_detect(m, cuts.p, nr * sc->n_sx, dmask.p, n_det, sc->n_sx, iy0,

@@ -60,7 +60,7 @@ template <int G>
 __global__ void __launch_bounds__(kCutWarps * 32, 2)
 k_exit_cut(const float2* __restrict__ S, int n_in, int nh, int m,
            const float2* __restrict__ axT, const float2* __restrict__ ayT, int n_sx, int n_sy,
-           const int* __restrict__ wx, const int* __restrict__ wy, int iy0,
+           const int* __restrict__ wx, const int* __restrict__ wy, int iy0, bool from_last,
            float2* __restrict__ out) {
   __shared__ ulonglong2 coef[2][kBeamChunk][G];   // (c.x, c.x), (c.y, c.y)
   __shared__ int dx[G];
@@ -68,10 +68,11 @@ k_exit_cut(const float2* __restrict__ S, int n_in, int nh, int m,
   const int np = min(G, n_sx - ix0);
   const int iyl = blockIdx.z;
   const int iy = iy0 + iyl;
-  // window origins on the grid (the block's row origin and first column origin decide
-  // for the whole block; a bad later column origin is replaced by the first)
-  if (!STEM_REQUIRE(wy[iy] >= 0 && wy[iy] < nh && wx[ix0] >= 0 && wx[ix0] < nh)) return;
-  const int xa = wx[ix0];
+  // columns are counted from the first probe's origin, or the last one's (from_last)
+  const int xa = wx[from_last ? ix0 + np - 1 : ix0];
+  // window origins on the grid (the block's row origin and that column origin decide for
+  // the whole block; a bad column origin of another probe is replaced by it)
+  if (!STEM_REQUIRE(wy[iy] >= 0 && wy[iy] < nh && xa >= 0 && xa < nh)) return;
   if (threadIdx.x < G) {
     int xg = threadIdx.x < np ? wx[ix0 + threadIdx.x] : xa;
     if (!STEM_REQUIRE(xg >= 0 && xg < nh)) xg = xa;
@@ -322,12 +323,13 @@ namespace {
 template <int G>
 cudaError_t exit_cut_g(const float2* S, int n_in, int nh, int m, const float2* axT,
                        const float2* ayT, int n_sx, int n_sy, const int* wx, const int* wy,
-                       int iy0, int n_rows, int max_span, float2* out, cudaStream_t s) {
+                       int iy0, int n_rows, int max_span, bool from_last, float2* out,
+                       cudaStream_t s) {
   const int elements = (m / 2) * std::min(m + max_span, nh), threads = kCutWarps * 32;
   dim3 g((unsigned)((n_sx + G - 1) / G), (unsigned)((elements + threads - 1) / threads),
          (unsigned)n_rows);
   k_exit_cut<G><<<g, kCutWarps * 32, 0, s>>>(S, n_in, nh, m, axT, ayT, n_sx, n_sy, wx, wy, iy0,
-                                             out);
+                                             from_last, out);
   return cudaGetLastError();
 }
 
@@ -335,16 +337,21 @@ cudaError_t exit_cut_g(const float2* S, int n_in, int nh, int m, const float2* a
 
 cudaError_t launch_exit_cut(const float2* S, int n_in, int nh, int m, const float2* axT,
                             const float2* ayT, int n_sx, int n_sy, const int* wx, const int* wy,
-                            int iy0, int n_rows, int max_span, float2* out, cudaStream_t s) {
+                            int iy0, int n_rows, int max_span, bool from_last, float2* out,
+                            cudaStream_t s) {
   if (n_rows <= 0) return cudaSuccess;
   // probes per CTA: 16 share each S value best; fewer where 16 would leave more than a
-  // quarter of the accumulators without a probe
+  // quarter of the accumulators without a probe, or half of the SMs without a CTA (64 x 64
+  // cuts of 16 x 2 probes, 145 beams: 102 us a call with 16 CTAs, 75 with 64)
   const int pad16 = (n_sx + 15) / 16 * 16, pad8 = (n_sx + 7) / 8 * 8;
-  if (n_sx <= 4)
-    return exit_cut_g<4>(S, n_in, nh, m, axT, ayT, n_sx, n_sy, wx, wy, iy0, n_rows, max_span, out, s);
-  if (4 * (pad16 - pad8) > pad16)
-    return exit_cut_g<8>(S, n_in, nh, m, axT, ayT, n_sx, n_sy, wx, wy, iy0, n_rows, max_span, out, s);
-  return exit_cut_g<16>(S, n_in, nh, m, axT, ayT, n_sx, n_sy, wx, wy, iy0, n_rows, max_span, out, s);
+  const int threads = kCutWarps * 32;
+  const int64_t per_group =
+      (int64_t)((m / 2 * std::min(m + max_span, nh) + threads - 1) / threads) * n_rows;
+  const auto fn = n_sx <= 4 || 2 * per_group * (pad8 / 8) < sm_count() ? exit_cut_g<4>
+                  : 4 * (pad16 - pad8) > pad16 || 2 * per_group * (pad16 / 16) < sm_count()
+                      ? exit_cut_g<8>
+                      : exit_cut_g<16>;
+  return fn(S, n_in, nh, m, axT, ayT, n_sx, n_sy, wx, wy, iy0, n_rows, max_span, from_last, out, s);
 }
 
 cudaError_t launch_cut_detect(int m, float2* X, int n_cut, const uint8_t* mask, int n_det,

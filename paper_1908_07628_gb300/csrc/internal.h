@@ -150,14 +150,15 @@ cudaError_t launch_accumulate(double* acc, const double* x, int64_t count, cudaS
 
 // Elastic images (elastic.cu).  Cut pass: out[r][sx][y'][x'] for scan rows iy0 ..
 // iy0 + n_rows - 1 = sum_j axT[sx][j] ayT[iy][j] S[j][(wy[iy] + y') % nh][(wx[sx] + x') % nh];
-// max_span: the largest cyclic distance of a column origin from that of an earlier probe
-// at most 15 positions before it.
+// max_span: the largest cyclic distance of a column origin from that of a probe at most 15
+// positions before it, or with from_last from that of one at most 15 positions after it.
 constexpr int kMaxDetectors = 8;
 constexpr int kMaxCutProbes = 16;   // probes of a scan row that one CTA may take
 bool cut_supported(int m);
 cudaError_t launch_exit_cut(const float2* S, int n_in, int nh, int m, const float2* axT,
                             const float2* ayT, int n_sx, int n_sy, const int* wx, const int* wy,
-                            int iy0, int n_rows, int max_span, float2* out, cudaStream_t s);
+                            int iy0, int n_rows, int max_span, bool from_last, float2* out,
+                            cudaStream_t s);
 // map[m][p] /= bf[p] for m < n_types, p < n_pix.
 cudaError_t launch_divide(double* map, const double* bf, int n_types, int64_t n_pix,
                           cudaStream_t s);
