@@ -886,10 +886,12 @@ eels_status map_window(eels_ctx* ctx, const eels_smatrix* sm, const eels_transit
   }
 
   // M buffer of the FP32 path, at most ~1 GiB of transitions: all types of a batch of
-  // sites, or some types of one site
+  // sites, or some types of one site; a launch's groups of 64 detector beams of all types
+  // fit the 65535 of a grid's second dimension
   const int64_t m_stride = (int64_t)n_out * n_in;
   const int64_t m_cap = std::max<int64_t>(1, ((int64_t)1 << 30) / (m_stride * (int64_t)sizeof(float2)));
-  const int fp_types = (int)std::min<int64_t>(T, m_cap);
+  const int fp_types = (int)std::min<int64_t>(
+      std::min<int64_t>(T, m_cap), std::max<int64_t>(1, 65535 / ((n_out + 63) / 64)));
   const int fp_sites = fp_types < T ? 1 : (int)std::min<int64_t>(
       std::min(std::max(max_sites, 1), 65535), m_cap / T);
   if (!tc) EELS_CK(M.alloc((size_t)fp_sites * fp_types * m_stride, st));
