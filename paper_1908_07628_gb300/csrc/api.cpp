@@ -1079,9 +1079,9 @@ eels_status map_window(eels_ctx* ctx, const eels_smatrix* sm, const eels_transit
   EELS_CK(axT.alloc((size_t)n_in * win.nx, st));
   EELS_CK(ayT.alloc((size_t)n_in * win.ny, st));
   EELS_CK(eels::launch_phase_table(axT.p, dbp.p, n_in, f, sm->cell, sc->x0, sc->step_x, win.nx,
-                                   st, 1, win.ix0));
+                                   st, win.ix0));
   EELS_CK(eels::launch_phase_table(ayT.p, dbq.p, n_in, f, sm->cell, sc->y0, sc->step_y, win.ny,
-                                   st, 1, win.iy0));
+                                   st, win.iy0));
 
   const eels::PlaneWaves plane_waves{dpx.p, dpy.p, damp.p};
   if (ctx->sout_scheme == EELS_SOUT_INVERSE) {
@@ -1553,9 +1553,9 @@ eels_status eels_elastic_images(eels_ctx* ctx, const eels_smatrix* sm, const eel
   EELS_CK(axT.alloc((size_t)n_in * sc->n_sx, st));
   EELS_CK(ayT.alloc((size_t)n_in * sc->n_sy, st));
   EELS_CK(eels::launch_phase_table(axT.p, dbp.p, n_in, f, sm->cell, sc->x0, sc->step_x, sc->n_sx,
-                                   st, 1));
+                                   st));
   EELS_CK(eels::launch_phase_table(ayT.p, dbq.p, n_in, f, sm->cell, sc->y0, sc->step_y, sc->n_sy,
-                                   st, 1));
+                                   st));
   // span of the column origins of probes that one CTA may take together, counted from the
   // first of them or (a scan towards smaller x) from the last
   int from_first = 0, from_last = 0;

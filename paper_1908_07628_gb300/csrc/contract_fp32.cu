@@ -289,11 +289,10 @@ k_gemm2_abs2(const float2* __restrict__ M, int64_t m_stride, int n_out, int n_in
 
 __global__ void k_phase_table(float2* __restrict__ out, const int* __restrict__ bidx, int n_beams,
                               int f, double cell, double r0, double step, int n_pos,
-                              int transposed, int r_first) {
+                              int r_first) {
   const int total = n_beams * n_pos;
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < total; i += gridDim.x * blockDim.x) {
-    const int j = transposed ? i % n_beams : i / n_pos;
-    const int r = transposed ? i / n_beams : i % n_pos;
+    const int j = i % n_beams, r = i / n_beams;
     const double R = __dadd_rn(r0, __dmul_rn((double)(r_first + r), step));
     double cyc = (double)f * (double)bidx[j] * R / cell;   // exp(-2 pi i cyc)
     cyc -= floor(cyc);
@@ -429,12 +428,12 @@ cudaError_t launch_gemm2_abs2_fp32(const float2* M, int64_t m_stride, int n_out,
 }
 
 cudaError_t launch_phase_table(float2* out, const int* bidx, int n_beams, int f, double cell,
-                               double r0, double step, int n_pos, cudaStream_t s, int transposed,
+                               double r0, double step, int n_pos, cudaStream_t s,
                                int r_first) {
   const int total = n_beams * n_pos;
   if (total <= 0) return cudaSuccess;
   k_phase_table<<<(total + 255) / 256, 256, 0, s>>>(out, bidx, n_beams, f, cell, r0, step, n_pos,
-                                                    transposed, r_first);
+                                                    r_first);
   return cudaGetLastError();
 }
 

@@ -169,7 +169,7 @@ k_cut_rows(float2* __restrict__ X, int64_t rows, const float2* __restrict__ tw) 
   constexpr int ROWS = RegFFT<M>::ROWS;
   constexpr int LDR = spad_len(M);
   constexpr int E = RegFFT<M>::E;
-  using PF = Plan<M, false>;
+  using PF = Plan<M>;
   extern __shared__ float2 smem[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   float2* sbuf = smem + warp * ROWS * LDR;
@@ -188,7 +188,7 @@ k_cut_rows(float2* __restrict__ X, int64_t rows, const float2* __restrict__ tw) 
         v[t * R0 + q] = live ? src[u % NB0 + q * NB0] : make_float2(0.f, 0.f);
     }
   }
-  reg_fft<M, false, false>(v, sbuf, LDR, tw, lane);
+  reg_fft<M>(v, sbuf, LDR, tw, lane);
   {
     constexpr int RF = PF::R(PF::NS - 1), NBF = M / RF, PERF = PF::per(PF::NS - 1);
 #pragma unroll
@@ -213,7 +213,7 @@ k_cut_cols_detect(const float2* __restrict__ X, const uint8_t* __restrict__ mask
   constexpr int ROWS = RegFFT<M>::ROWS;
   constexpr int LDR = spad_len(M);
   constexpr int E = RegFFT<M>::E;
-  using PF = Plan<M, false>;
+  using PF = Plan<M>;
   extern __shared__ float2 smem[];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   float2* sbuf = smem + warp * ROWS * LDR;
@@ -233,7 +233,7 @@ k_cut_cols_detect(const float2* __restrict__ X, const uint8_t* __restrict__ mask
         v[t * R0 + q] = live ? cut[(int64_t)(u % NB0 + q * NB0) * M + col] : make_float2(0.f, 0.f);
     }
   }
-  reg_fft<M, false, false>(v, sbuf, LDR, tw, lane);
+  reg_fft<M>(v, sbuf, LDR, tw, lane);
   float acc[kMaxDetectors];
 #pragma unroll
   for (int d = 0; d < kMaxDetectors; ++d) acc[d] = 0.f;

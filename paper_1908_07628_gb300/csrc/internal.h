@@ -129,12 +129,11 @@ cudaError_t launch_gemm2_abs2_fp32(const float2* M, int64_t m_stride, int n_out,
                                    const float2* axT, const float2* ayT, int n_sx, int n_sy,
                                    const SiteBatch& sb, const WindowLists& wl, double* map,
                                    cudaStream_t s);
-// ax[j][ix] = exp(-2 pi i f p_j Rx(ix) / L) (FP64 phase); same for ay with q_j, Ry.  Row
+// axT[ix][j] = exp(-2 pi i f p_j Rx(ix) / L) (FP64 phase); same for ayT with q_j, Ry.  Row
 // ix holds position Rx = r0 + (r_first + ix) step (a window of a longer scan line).
-// transposed = 1 writes out[pos][j] instead (coalesced reads along the beams).
 cudaError_t launch_phase_table(float2* out, const int* bidx, int n_beams, int f, double cell,
                                double r0, double step, int n_pos, cudaStream_t s,
-                               int transposed = 0, int r_first = 0);
+                               int r_first = 0);
 cudaError_t launch_scale(double* a, int64_t count, double scale, cudaStream_t s);
 // a *= scale; bit 2 of *flag is set if any result is NaN or Inf (the map's sentinel)
 cudaError_t launch_scale_check(double* a, int64_t count, double scale, int* flag,

@@ -712,13 +712,10 @@ void fill_twiddle_tables(int n, float2* h) {
   if (grid_supported(n))
     for (int i = 0; i < 4; ++i) fill_plan_set(n, i >= 2, i & 1, h);
   if (plan_len(n) != 2) return;
-  for (int rev = 0; rev < 2; ++rev) {
-    // stage 1 of the plan: radix r1 after a first stage of radix r0 (r0 r1 = n)
-    const int r0 = plan_radix(n, rev ? 1 : 0), r1 = plan_radix(n, rev ? 0 : 1);
-    float2* t = h + twiddle_table_offset(n, rev != 0);
-    for (int q = 0; q < r1; ++q)
-      for (int k = 0; k < r0; ++k) t[q * r0 + k] = root((int64_t)q * k);
-  }
+  // stage 1 of the two-stage plan: radix r1 after a first stage of radix r0 (r0 r1 = n)
+  const int r0 = plan_radix(n, 0), r1 = plan_radix(n, 1);
+  for (int q = 0; q < r1; ++q)
+    for (int k = 0; k < r0; ++k) h[n + q * r0 + k] = root((int64_t)q * k);
 }
 
 cudaError_t launch_row_pass(int n, int n_waves, const float2* W, float2* Phi, const float2* t,
