@@ -7,7 +7,7 @@
 // kx' - N/2).  Because the propagator limits every wave to p^2 + q^2 < (N/4)^2,
 // nothing outside the box is ever needed.
 //
-//   row pass    (one warp per row y):  zero-pad kx to N, inverse FFT_x, multiply
+//   row pass    (one warp per 1, 2 or 4 rows y): zero-pad kx to N, inverse FFT_x, multiply
 //                by t (or conj t), optionally store the even samples (the N/2
 //                representation used by the S-matrices), forward FFT_x, keep the box.
 //   column pass (one CTA per few columns kx'): FFT_y, keep the box, multiply by the
@@ -141,13 +141,16 @@ __device__ __forceinline__ void row_wave(float2* v, float2* sbuf, const float2* 
   }
 }
 
-// Row pass.  A CTA takes SEQ rows y0 .. y0 + SEQ - 1 of `chunk` waves, one warp a wave at a
-// time: the rows of t and the factor sets lie in shared memory for all of them (read per
-// row from L2 and L1 they cost as many wavefronts and far more latency), and the rows of a
-// warp's next wave are fetched to L2 while it transforms this one's.  Bound by issue slots
-// (ncu, 1024: 69 %, FMA pipe 55 %, shared-memory wavefronts 66 %, DRAM 45 %).  Adjoint pass
-// with the S_out store, us per wave, before -> now: 1024: 3.22 -> 2.95, 768: 1.83 -> 1.55,
-// 512: 0.58 -> 0.57, 384: 1.00 -> 0.48 (four stages and three exchanges before).
+// Row pass of many waves.  A CTA takes SEQ rows y0 .. y0 + SEQ - 1 of `chunk` waves, one warp
+// a wave at a time: the rows of t and the factor sets lie in shared memory for all of them
+// (read per row from L2 and L1 they cost as many wavefronts and far more latency), and the
+// rows of a warp's next wave are fetched to L2 while it transforms this one's.  No unit is
+// saturated: of the issue slots 68 % are used (ncu, 305 waves at 1024; L1 and shared memory
+// 68 %, FMA pipe 55 %, DRAM 45 %), one warp in six waits for instructions, and 16 warps are
+// what the registers allow.  us per wave, rows read per wave / so: adjoint pass with the
+// S_out store, 1024: 3.22 / 2.95, 768: 1.83 / 1.55, 512: 0.58 / 0.57, 384: 1.00 / 0.48 (four
+// stages and three exchanges before); pass of a build, 256: 0.150 / 0.146, 128: 0.085 / 0.043,
+// 64: 0.036 / 0.018.
 template <int N, bool CONJ, bool START>
 __global__ void __launch_bounds__(kRowWarps * 32, row_ctas<N>())
 k_row_pass(const float2* __restrict__ W, const PlaneWaves start, float2* __restrict__ Phi,

@@ -325,7 +325,8 @@ __device__ __forceinline__ void super_stage(float2* v, int k, const float2* ta, 
 // x_{u / NB0}[u % NB0 + q N/R0] at v[t R0 + q], on exit X in the same form for R1 and NB1.
 // Sequence r exchanges through sbuf + r * ld (PADDED values; a first super-stage writes
 // R0 b + o into rows of R0 + 1 values, so that neighbouring lanes hit distinct banks).
-// `set` is the factor set of the plan, in shared memory (load_set).
+// `set` is the part of the factor set that the plan reads (SetPart), in shared memory
+// (load_sets) or in the table itself.
 template <int N, bool INV, bool REV, bool EDGE>
 __device__ __forceinline__ void warp_fft(float2* v, float2* sbuf, int ld, const float2* set,
                                          int lane) {
