@@ -540,10 +540,10 @@ k_tc_gemm_ws(const __grid_constant__ CUtensorMap ta, const __grid_constant__ CUt
   if (!ok && status) atomicExch(status, 1);
 }
 
-// Window gathers: a warp takes one beam's window, or one batch of it where gridDim.z is the
-// number of batches (window_grid), its lanes pixel pairs p, p + 1 (p = 2 lane, then steps of
-// 64).  The pair's window row and column advance by fixed steps (no division), and each batch
-// of kPairBatch pairs is loaded before any of its stores.
+// Window gathers: a warp takes one beam's window, or with SPREAD the batch blockIdx.z of it
+// (spread_batches), its lanes pixel pairs p, p + 1 (p = 2 lane, then steps of 64).  The pair's
+// window row and column advance by fixed steps (no division), and each batch of kPairBatch
+// pairs is loaded before any of its stores.
 constexpr int kPairBatch = 4;
 
 struct PairWalk {
@@ -604,7 +604,7 @@ constexpr int kArowRows = 16;     // probe rows per block of the probe-row gathe
 // A1[slot][plane][d][2p + c] = Sout[d][pixel p of the window of site slot_site[slot]].
 // (A block per four beams with single pixels stored 4 bytes at a time in BF16 and left most
 // of a 24-pixel window's last batch of loads empty: 57 % of the copy bandwidth.)
-template <int PREC>
+template <int PREC, bool SPREAD>
 __global__ void __launch_bounds__(kGatherBeams * 32)
 k_gather_sout(const float2* __restrict__ Sout, int nh, int n_out, int w,
               const int* __restrict__ slot_site, const int* __restrict__ wx,
@@ -618,19 +618,20 @@ k_gather_sout(const float2* __restrict__ Sout, int nh, int n_out, int w,
   const int64_t row = (int64_t)slot * PL * pstride + (int64_t)d * k1p;
   const float2* src = Sout + (int64_t)d * nh * nh;
   const int P = w * w;
-  int p = 2 * (threadIdx.x & 31) + 64 * kPairBatch * blockIdx.z;
+  int p = 2 * (threadIdx.x & 31) + (SPREAD ? 64 * kPairBatch * blockIdx.z : 0);
   PairWalk walk(wx[s], wy[s], w, nh, p);
-  for (; p < k1p / 2; p += 64 * kPairBatch * gridDim.z) {   // up to the K padding, which is zero
+  for (; p < k1p / 2; p += 64 * kPairBatch) {   // up to the K padding, which is zero
     float2 v[kPairBatch][2];
     walk.load(src, p, P, v);
 #pragma unroll
     for (int u = 0; u < kPairBatch; ++u)
       if (p + 64 * u < k1p / 2) put4<PREC>(A1, pstride, row + 2 * (p + 64 * u), v[u][0], v[u][1]);
+    if (SPREAD) break;
   }
 }
 
 // B1[z][plane][2j][2p + c] = H_z[p] Sin[j][p],  B1[z][plane][2j+1] = -i H_z[p] Sin[j][p]
-template <int PREC>
+template <int PREC, bool SPREAD>
 __global__ void __launch_bounds__(kGatherBeams * 32)
 k_gather_sin_h(const float2* __restrict__ Sin, int nh, int n_in, int w,
                const int* __restrict__ z_site, const int* __restrict__ z_type,
@@ -650,9 +651,9 @@ k_gather_sin_h(const float2* __restrict__ Sin, int nh, int n_in, int w,
   const int P = w * w;
   const float2* Hz = H + ((int64_t)s * h_mul * n_types + z_type[z]) * P;
   const float2* src = Sin + (int64_t)j * nh * nh;
-  int p = 2 * (threadIdx.x & 31) + 64 * kPairBatch * blockIdx.z;
+  int p = 2 * (threadIdx.x & 31) + (SPREAD ? 64 * kPairBatch * blockIdx.z : 0);
   PairWalk walk(wx[s], wy[s], w, nh, p);
-  for (; p < k1p / 2; p += 64 * kPairBatch * gridDim.z) {
+  for (; p < k1p / 2; p += 64 * kPairBatch) {
     float2 v[kPairBatch][2];
     walk.load(src, p, P, v);
 #pragma unroll
@@ -666,6 +667,7 @@ k_gather_sin_h(const float2* __restrict__ Sin, int nh, int n_in, int w,
       put4<PREC>(B1, pstride, r0 + 2 * q, y[0], y[1]);
       put4<PREC>(B1, pstride, r1 + 2 * q, make_float2(y[0].y, -y[0].x), make_float2(y[1].y, -y[1].x));
     }
+    if (SPREAD) break;
   }
 }
 
@@ -858,24 +860,37 @@ cudaError_t gather_arows_impl(const TcBatch& b, const int* site, int count, cuda
   return cudaGetLastError();
 }
 
-// Grid of a gather of `beams` beams in `n` windows.  A warp that takes a window's batches one
-// after another waits for each; where the launch has fewer than 16 CTAs per SM the batches
-// are spread over gridDim.z instead.  89 + 37 beams, 32 windows of 32 x 32 pixels, TF32: 37.4
-// us in order, 30.5 spread; 1321 beams, 128 windows of 26 x 26: 823 in order, 840 spread.
-dim3 window_grid(int beams, int n, int k1p) {
-  const int bx = (beams + kGatherBeams - 1) / kGatherBeams;
-  const int batches = (k1p / 2 + 64 * kPairBatch - 1) / (64 * kPairBatch);
-  return dim3(bx, n, (int64_t)bx * n < 16 * sm_count() ? batches : 1);
+// A gather of `beams` beams in `n` windows: 0, a warp takes a window's batches one after another
+// and waits for each, or where the launch would have fewer than 16 CTAs per SM the number of
+// batches, to be spread over gridDim.z.  89 + 37 beams, 32 windows of 32 x 32 pixels, TF32:
+// 37.4 us in order, 30.5 spread; 1321 beams, 128 windows of 26 x 26: 823 in order, 840
+// spread.
+int spread_batches(int beams, int n, int k1p) {
+  const int64_t ctas = (int64_t)((beams + kGatherBeams - 1) / kGatherBeams) * n;
+  return ctas < 16 * sm_count() ? (k1p / 2 + 64 * kPairBatch - 1) / (64 * kPairBatch) : 0;
+}
+dim3 window_grid(int beams, int n, int batches) {
+  return dim3((beams + kGatherBeams - 1) / kGatherBeams, n, std::max(batches, 1));
+}
+
+// S_out windows of the batch's sites (A1)
+template <int PREC>
+cudaError_t gather_sout_impl(const TcBatch& b, cudaStream_t st) {
+  const int z = spread_batches(b.n_out, b.n_sites, b.k1p);
+  const auto kernel = z ? k_gather_sout<PREC, true> : k_gather_sout<PREC, false>;
+  kernel<<<window_grid(b.n_out, b.n_sites, z), 256, 0, st>>>(b.Sout, b.nh, b.n_out, b.w, b.slot_site,
+                                                             b.wx, b.wy, b.A1, b.k1p);
+  return cudaGetLastError();
 }
 
 template <int PREC>
 cudaError_t gather_impl(const TcBatch& b, cudaStream_t st) {
   const int nz = b.n_sites * b.n_types;
   cudaError_t e;
-  k_gather_sout<PREC><<<window_grid(b.n_out, b.n_sites, b.k1p), 256, 0, st>>>(
-      b.Sout, b.nh, b.n_out, b.w, b.slot_site, b.wx, b.wy, b.A1, b.k1p);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
-  k_gather_sin_h<PREC><<<window_grid(b.n_in, nz, b.k1p), 256, 0, st>>>(
+  if ((e = gather_sout_impl<PREC>(b, st)) != cudaSuccess) return e;
+  const int z = spread_batches(b.n_in, nz, b.k1p);
+  const auto kernel = z ? k_gather_sin_h<PREC, true> : k_gather_sin_h<PREC, false>;
+  kernel<<<window_grid(b.n_in, nz, z), 256, 0, st>>>(
       b.Sin, b.nh, b.n_in, b.w, b.z_site, b.z_type, b.H, b.n_types, b.h_mul, b.wx, b.wy, b.B1, b.k1p);
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
   return b.n_sets ? cudaSuccess : gather_probe_impl<PREC>(b, b.slot_site, b.n_sites, st);
@@ -947,9 +962,7 @@ cudaError_t gemm2_impl(const TcBatch& b, cudaStream_t st) {
 template <int PREC>
 cudaError_t gather_y_impl(const TcBatch& b, cudaStream_t st) {
   cudaError_t e;
-  k_gather_sout<PREC><<<window_grid(b.n_out, b.n_sites, b.k1p), 256, 0, st>>>(
-      b.Sout, b.nh, b.n_out, b.w, b.slot_site, b.wx, b.wy, b.A1, b.k1p);
-  if ((e = cudaGetLastError()) != cudaSuccess) return e;
+  if ((e = gather_sout_impl<PREC>(b, st)) != cudaSuccess) return e;
   if (!b.n_sets && (e = gather_arows_impl<PREC>(b, b.slot_site, b.n_sites, st)) != cudaSuccess)
     return e;
   dim3 gt((b.k1p / 2 + 31) / 32, (b.k2p / 2 + 31) / 32, b.n_sites);
