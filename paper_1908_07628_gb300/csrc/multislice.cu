@@ -187,8 +187,8 @@ k_row_pass(const float2* __restrict__ W, const PlaneWaves start, float2* __restr
 
 // Row pass of few waves: a warp takes SEQ rows of one wave and the CTA's warps neighbouring
 // rows; t and the factor sets are read where they lie (L2, L1) and no warp waits for another.
-// Where a warp has one or two waves, k_row_pass spends as long on filling shared memory as
-// on a wave, and of the 4 m + 1 beams of an aperture three warps of the last CTA have none.
+// k_row_pass fills shared memory before its first butterfly, which one or two waves a warp do
+// not pay for, and of the 4 m + 1 beams of an aperture three warps of its last CTA have none.
 // Mean row launch of a build, us, k_row_pass -> this: 512: 9 waves 16.2 -> 12.4, 37 34.7 ->
 // 30.5; 256: 37 13.9 -> 12.3; 1024: 5 28.3 -> 24.5; 768: 9 28.4 -> 23.8; 128: 37 8.3 -> 8.2.
 // Six CTAs per SM at 256 (80 registers): 145 waves 28.5 us, with five 30.0.
@@ -535,9 +535,10 @@ int wave_chunk(int n_waves, int blocks_x, int width, int resident) {
 }
 
 // The chunk between half and twice of `chunk` (at most 16) whose rounds of CTAs, two to an
-// SM, take least, the largest of equal ones.  A last round of at most one CTA per SM takes
-// about 0.6 of a full one.  512 columns pass: 593 waves in chunks of 10 leave a fourth round
-// of 48 CTAs, in chunks of 16 two full rounds.
+// SM, take least, the largest of equal ones.  A last round of at most one CTA per SM, which
+// then has it to itself, is counted as 0.6 of a full one (an estimate).  Pass at 512: 593
+// waves in chunks of 10 leave a fourth round of 48 CTAs, in chunks of 16 two full rounds; 145
+// waves 80 us with chunks of 5, 70 so, 441 waves 219 and 182; at 768 1329 waves 1441 and 1411.
 int even_rounds(int n_waves, int blocks_x, int chunk) {
   const int64_t sms = sm_count();
   int best = chunk;
